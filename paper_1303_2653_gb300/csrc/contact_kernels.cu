@@ -15,8 +15,9 @@
 // the particle spins; the spins after the step are written for the sort to
 // carry, those of the start of the step are read.
 //
-// One thread per particle in sorted order, walking the cells within reach
-// (as the hard-sphere detection does).  The separation of a pair is formed in
+// One thread per particle in sorted order: in sparse beds it walks the cells
+// within reach (as the hard-sphere detection does), in crowded ones a block
+// bins the particles around its own in shared memory.  The separation of a pair is formed in
 // the arithmetic type from the cell indices and in-cell offsets; only a pair
 // whose squared distance lies within a thin band around d^2 (wider than the
 // rounding of the offsets) takes the exact FP64 test on the positions that
@@ -31,47 +32,6 @@ namespace lbdpsk {
 template <int D, class Real, bool FRIC> struct ContactOccupancy { static constexpr int value = 2; };
 template <> struct ContactOccupancy<2, float, false> { static constexpr int value = 6; };
 template <> struct ContactOccupancy<2, float, true> { static constexpr int value = 5; };
-
-// Tangential (friction) part of one contact seen from particle i: unit normal
-// n towards i, lever arm l from i's centre to the contact point (at -l n),
-// clipped normal force fn > 0, relative velocity of the contact point vc
-// (i's minus the other body's, three components, z only used in 3D).  The
-// slip v_t = vc - (vc.n) n meets -min(gamma_t |v_t|, mu fn) v_t / |v_t|,
-// added to F; its torque (-l n) x F_t is added to T (T[0] holds the
-// component normal to the plane in 2D).
-template <int D, class Real>
-__device__ __forceinline__ void friction(const StepParams<Real> &p, const Real *n, Real l, Real fn,
-                                         const Real *vc, Real *F, Real *T)
-{
-    Real vcn = Real(0);
-#pragma unroll
-    for (int a = 0; a < D; ++a) vcn += vc[a] * n[a];
-    Real vt[3] = {Real(0), Real(0), Real(0)}, s2 = Real(0);
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        vt[a] = vc[a] - vcn * n[a];
-        s2 += vt[a] * vt[a];
-    }
-    if (!(s2 > Real(0))) return;
-    const Real st = sqrt(s2);
-    Real mag = p.gamma_t * st;
-    const Real cap = p.mu_f * fn;
-    if (mag > cap) mag = cap;
-    const Real k = -mag / st;
-    Real Ft[3] = {Real(0), Real(0), Real(0)};
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        Ft[a] = k * vt[a];
-        F[a] += Ft[a];
-    }
-    if (D == 2) {
-        T[0] -= l * (n[0] * Ft[1] - n[1] * Ft[0]);
-    } else {
-        T[0] -= l * (n[1] * Ft[2] - n[2] * Ft[1]);
-        T[1] -= l * (n[2] * Ft[0] - n[0] * Ft[2]);
-        T[2] -= l * (n[0] * Ft[1] - n[1] * Ft[0]);
-    }
-}
 
 // w x n for the spin w (one component normal to the plane in 2D) and an
 // in-plane (2D) or 3D vector n
@@ -89,98 +49,128 @@ __device__ __forceinline__ void spin_cross(const Real *w, const Real *n, Real *o
     }
 }
 
-// FRIC: soft spheres with friction (spins read from parts.w, the new spins
-// written to p.spin_out)
+// One contact as it acts on particle i: unit normal n towards i and normal
+// force f > 0; with friction also the tangential force Ft, the lever arm l from
+// i's centre to the contact point (at -l n) and n x Ft (cr[0] holds the
+// component normal to the plane in 2D), so that the torque is -l cr.
+template <class Real, bool FRIC> struct Push;
+template <class Real> struct Push<Real, false> { Real f, n[3]; };
+template <class Real> struct Push<Real, true> { Real f, n[3], Ft[3], l, cr[3]; };
+
+// Adds a contact to the force F and the torque T.
 template <int D, class Real, bool FRIC>
-__global__ void __launch_bounds__(256, ContactOccupancy<D, Real, FRIC>::value)
-k_contacts(StepParams<Real> p, Particles<Real> parts, CellList cells, Real *diag_fc, int np)
+__device__ __forceinline__ void add_push(const Push<Real, FRIC> &c, Real *F, Real *T)
 {
-    constexpr int NW = D == 2 ? 1 : 3;   // spin components
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= np) return;
-    int idx[3];
-    cell_coords(D, p.n, __ldg(parts.cell + i), idx);
-    float oi[3] = {0.f, 0.f, 0.f};
-    Real vi[3] = {Real(0), Real(0), Real(0)}, wi[3] = {Real(0), Real(0), Real(0)};
-    bool per[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        per[a] = (a < D) && (p.bc[2 * a] == BC_PERIODIC);
-        if (a < D) {
-            oi[a] = (float)__ldg(parts.off[a] + i);
-            vi[a] = __ldg(parts.v[a] + i);
-        }
-    }
-    if (FRIC) {
+    for (int a = 0; a < D; ++a) F[a] += c.f * c.n[a];
+    if constexpr (FRIC) {
 #pragma unroll
-        for (int c = 0; c < NW; ++c) wi[c] = __ldg(parts.w[c] + i);
+        for (int a = 0; a < D; ++a) F[a] += c.Ft[a];
+#pragma unroll
+        for (int k = 0; k < (D == 2 ? 1 : 3); ++k) T[k] -= c.l * c.cr[k];
     }
-    const float cut = (float)p.d + 1e-4f;   // reach of the walk
-    // squared distances beyond d2_hi cannot be contacts, those below d2_lo
-    // are; the band between covers the rounding of the offsets (about 1e-7
-    // in FP32 on a separation of at most 2)
-    const Real band = sizeof(Real) == 4 ? Real(4e-6) : Real(1e-12);
+}
+
+// Tangential (friction) part of a contact (c.f, c.n and c.l set), from the
+// relative velocity vc of the contact point (i's minus the other body's, three
+// components, z only used in 3D).  The slip v_t = vc - (vc.n) n meets
+// -min(gamma_t |v_t|, mu f) v_t / |v_t|.
+template <int D, class Real>
+__device__ __forceinline__ void friction(const StepParams<Real> &p, const Real *vc,
+                                         Push<Real, true> &c)
+{
+#pragma unroll
+    for (int a = 0; a < 3; ++a) c.Ft[a] = c.cr[a] = Real(0);
+    Real vcn = Real(0);
+#pragma unroll
+    for (int a = 0; a < D; ++a) vcn += vc[a] * c.n[a];
+    Real vt[3] = {Real(0), Real(0), Real(0)}, s2 = Real(0);
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        vt[a] = vc[a] - vcn * c.n[a];
+        s2 += vt[a] * vt[a];
+    }
+    if (!(s2 > Real(0))) return;
+    const Real st = sqrt(s2);
+    Real mag = p.gamma_t * st;
+    const Real cap = p.mu_f * c.f;
+    if (mag > cap) mag = cap;
+    const Real k = -mag / st;
+#pragma unroll
+    for (int a = 0; a < D; ++a) c.Ft[a] = k * vt[a];
+    if (D == 2) {
+        c.cr[0] = c.n[0] * c.Ft[1] - c.n[1] * c.Ft[0];
+    } else {
+        c.cr[0] = c.n[1] * c.Ft[2] - c.n[2] * c.Ft[1];
+        c.cr[1] = c.n[2] * c.Ft[0] - c.n[0] * c.Ft[2];
+        c.cr[2] = c.n[0] * c.Ft[1] - c.n[1] * c.Ft[0];
+    }
+}
+
+// Squared distances beyond d^2 + band cannot be contacts, those below d^2 -
+// band are; the band between covers the rounding of the offsets (about 1e-7
+// in FP32 on a separation of at most 2).
+template <class Real> __device__ __forceinline__ Real contact_band()
+{
+    return sizeof(Real) == 4 ? Real(4e-6) : Real(1e-12);
+}
+
+// The contact of particles i and j whose separation dx (i minus j, squared
+// length d2 <= d^2 + band) is known, as it acts on i.  False for a pair that
+// does not push.  vi, wi: i's velocity and spin.
+template <int D, class Real, bool FRIC>
+__device__ __forceinline__ bool pair_push(const StepParams<Real> &p, const Particles<Real> &parts,
+                                          int i, int j, const bool *per, const Real *dx, Real d2,
+                                          const Real *vi, const Real *wi, Push<Real, FRIC> &c)
+{
     const Real dd = (Real)p.d2;
-    const Real d2_lo = dd - band, d2_hi = dd + band;
-    Real oR[3] = {Real(0), Real(0), Real(0)};
-#pragma unroll
-    for (int a = 0; a < D; ++a) oR[a] = __ldg(parts.off[a] + i);
-    Real F[3] = {Real(0), Real(0), Real(0)}, T[3] = {Real(0), Real(0), Real(0)};
-
-    auto pair = [&](int j, int rowbase, float sy, float sz) {
-        if (j == i) return;
-        const Real shift[3] = {(Real)x_shift(p, parts, idx, per[0], j, rowbase), (Real)sy, (Real)sz};
-        Real dx[3] = {Real(0), Real(0), Real(0)};
-        Real d2 = Real(0);
+    if (!(d2 < dd - contact_band<Real>())) {
+        // near the contact distance: the exact test of the oracle
+        double e2 = 0.0;
 #pragma unroll
         for (int a = 0; a < D; ++a) {
-            dx[a] = oR[a] - __ldg(parts.off[a] + j) - shift[a];
-            d2 += dx[a] * dx[a];
+            const double t = sep_axis(__ldg(parts.P[a] + i), __ldg(parts.P[a] + j), per[a], p.len[a]);
+            e2 = __dadd_rn(e2, __dmul_rn(t, t));
         }
-        if (d2 > d2_hi) return;
-        if (!(d2 < d2_lo)) {
-            // near the contact distance: the exact test of the oracle
-            double e2 = 0.0;
+        if (!(e2 < p.d2)) return false;
+        if (d2 >= dd) d2 = dd;   // the overlap is then below the rounding: zero
+    }
+    const Real dist = sqrt(d2);
+    const Real delta = (dd - d2) / ((Real)p.d + dist);
+    Real vr[3] = {Real(0), Real(0), Real(0)};
+    Real vn = Real(0);
 #pragma unroll
-            for (int a = 0; a < D; ++a) {
-                const double t = sep_axis(__ldg(parts.P[a] + i), __ldg(parts.P[a] + j), per[a], p.len[a]);
-                e2 = __dadd_rn(e2, __dmul_rn(t, t));
-            }
-            if (!(e2 < p.d2)) return;
-            if (d2 >= dd) d2 = dd;   // the overlap is then below the rounding: zero
-        }
-        const Real dist = sqrt(d2);
-        const Real delta = (dd - d2) / ((Real)p.d + dist);
-        Real nrm[3] = {Real(0), Real(0), Real(0)}, vr[3] = {Real(0), Real(0), Real(0)};
-        Real vn = Real(0);
+    for (int a = 0; a < D; ++a) {
+        c.n[a] = dx[a] / dist;
+        vr[a] = vi[a] - __ldg(parts.v[a] + j);
+        vn += vr[a] * c.n[a];
+    }
+    c.f = p.kn * delta - p.eta * vn;
+    if (!(c.f > Real(0))) return false;
+    if constexpr (FRIC) {
+        // contact point half way: vc = v_rel - l (w_i + w_j) x n
+        c.l = Real(0.5) * dist;
+        Real ws[3] = {Real(0), Real(0), Real(0)}, wxn[3], vc[3];
 #pragma unroll
-        for (int a = 0; a < D; ++a) {
-            nrm[a] = dx[a] / dist;
-            vr[a] = vi[a] - __ldg(parts.v[a] + j);
-            vn += vr[a] * nrm[a];
-        }
-        const Real f = p.kn * delta - p.eta * vn;
-        if (f > Real(0)) {
+        for (int k = 0; k < (D == 2 ? 1 : 3); ++k) ws[k] = wi[k] + __ldg(parts.w[k] + j);
+        spin_cross<D, Real>(ws, c.n, wxn);
 #pragma unroll
-            for (int a = 0; a < D; ++a) F[a] += f * nrm[a];
-            if (FRIC) {
-                // contact point half way: vc = v_rel - l (w_i + w_j) x n
-                const Real l = Real(0.5) * dist;
-                Real ws[3] = {Real(0), Real(0), Real(0)}, wxn[3], vc[3];
-#pragma unroll
-                for (int c = 0; c < NW; ++c) ws[c] = wi[c] + __ldg(parts.w[c] + j);
-                spin_cross<D, Real>(ws, nrm, wxn);
-#pragma unroll
-                for (int a = 0; a < 3; ++a) vc[a] = vr[a] - l * wxn[a];
-                friction<D, Real>(p, nrm, l, f, vc, F, T);
-            }
-        }
-    };
-    visit_neighbours<D, Real>(p, cells, idx, per, oi, cut, pair);
+        for (int a = 0; a < 3; ++a) vc[a] = vr[a] - c.l * wxn[a];
+        friction<D, Real>(p, vc, c);
+    }
+    return true;
+}
 
-    // faces: only the first and last cell of an axis can be within r < 1/2
-    // of one; the open outlet of a circulating bed makes no contact.  The
-    // contact point lies on the face, at the centre's distance from it.
+// The faces' part of particle i (only the first and last cell of an axis can
+// be within r < 1/2 of one; the open outlet of a circulating bed makes no
+// contact; the contact point lies on the face, at the centre's distance from
+// it), added to F and T, and the step's results of the particle.
+template <int D, class Real, bool FRIC>
+__device__ __forceinline__ void finish_contacts(const StepParams<Real> &p,
+                                                const Particles<Real> &parts, int i, const int *idx,
+                                                const bool *per, const Real *vi, const Real *wi,
+                                                Real *F, Real *T, Real *diag_fc, int np)
+{
 #pragma unroll
     for (int a = 0; a < D; ++a) {
         if (per[a]) continue;
@@ -195,14 +185,20 @@ k_contacts(StepParams<Real> p, Particles<Real> parts, CellList cells, Real *diag
             const Real f = p.kn * (Real)__dsub_rn(p.r64, gap) - p.eta_w * (sg * vi[a]);
             if (!(f > Real(0))) continue;
             F[a] += sg * f;
-            if (FRIC) {
-                Real nrm[3] = {Real(0), Real(0), Real(0)}, wxn[3], vc[3];
-                nrm[a] = sg;
-                const Real l = (Real)gap;
-                spin_cross<D, Real>(wi, nrm, wxn);
+            if constexpr (FRIC) {
+                Push<Real, true> c{};
+                c.f = f;
+                c.n[a] = sg;
+                c.l = (Real)gap;
+                Real wxn[3], vc[3];
+                spin_cross<D, Real>(wi, c.n, wxn);
 #pragma unroll
-                for (int c = 0; c < 3; ++c) vc[c] = vi[c] - l * wxn[c];
-                friction<D, Real>(p, nrm, l, f, vc, F, T);
+                for (int k = 0; k < 3; ++k) vc[k] = vi[k] - c.l * wxn[k];
+                friction<D, Real>(p, vc, c);
+#pragma unroll
+                for (int k = 0; k < D; ++k) F[k] += c.Ft[k];
+#pragma unroll
+                for (int k = 0; k < (D == 2 ? 1 : 3); ++k) T[k] -= c.l * c.cr[k];
             }
         }
     }
@@ -211,7 +207,7 @@ k_contacts(StepParams<Real> p, Particles<Real> parts, CellList cells, Real *diag
     if (FRIC) {
         // I dw = T dt from the start-of-step state
 #pragma unroll
-        for (int c = 0; c < NW; ++c) p.spin_out[c][i] = wi[c] + T[c] * p.inv_inertia;
+        for (int k = 0; k < (D == 2 ? 1 : 3); ++k) p.spin_out[k][i] = wi[k] + T[k] * p.inv_inertia;
     }
     if (diag_fc) {
         const int id = parts.id[i];
@@ -220,18 +216,448 @@ k_contacts(StepParams<Real> p, Particles<Real> parts, CellList cells, Real *diag
     }
 }
 
+// One thread per particle (sparse beds): each walks the cells within its own
+// reach.  FRIC: soft spheres with friction (spins read from parts.w, the new
+// spins written to p.spin_out).
+template <int D, class Real, bool FRIC>
+__global__ void __launch_bounds__(256, ContactOccupancy<D, Real, FRIC>::value)
+k_contacts(StepParams<Real> p, Particles<Real> parts, CellList cells, Real *diag_fc, int np)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= np) return;
+    int idx[3];
+    cell_coords(D, p.n, __ldg(parts.cell + i), idx);
+    float oi[3] = {0.f, 0.f, 0.f};
+    Real oR[3] = {Real(0), Real(0), Real(0)};
+    Real vi[3] = {Real(0), Real(0), Real(0)}, wi[3] = {Real(0), Real(0), Real(0)};
+    bool per[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        per[a] = (a < D) && (p.bc[2 * a] == BC_PERIODIC);
+        if (a < D) {
+            oR[a] = __ldg(parts.off[a] + i);
+            oi[a] = (float)oR[a];
+            vi[a] = __ldg(parts.v[a] + i);
+        }
+    }
+    if (FRIC) {
+#pragma unroll
+        for (int c = 0; c < (D == 2 ? 1 : 3); ++c) wi[c] = __ldg(parts.w[c] + i);
+    }
+    const float cut = (float)p.d + 1e-4f;   // reach of the walk
+    const Real d2_hi = (Real)p.d2 + contact_band<Real>();
+    Real F[3] = {Real(0), Real(0), Real(0)}, T[3] = {Real(0), Real(0), Real(0)};
+
+    auto pair = [&](int j, int rowbase, float sy, float sz) {
+        if (j == i) return;
+        const Real shift[3] = {(Real)x_shift(p, parts, idx, per[0], j, rowbase), (Real)sy, (Real)sz};
+        Real dx[3] = {Real(0), Real(0), Real(0)};
+        Real d2 = Real(0);
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            dx[a] = oR[a] - __ldg(parts.off[a] + j) - shift[a];
+            d2 += dx[a] * dx[a];
+        }
+        if (d2 > d2_hi) return;
+        Push<Real, FRIC> c;
+        if (pair_push<D, Real, FRIC>(p, parts, i, j, per, dx, d2, vi, wi, c))
+            add_push<D, Real, FRIC>(c, F, T);
+    };
+    visit_neighbours<D, Real>(p, cells, idx, per, oi, cut, pair);
+    finish_contacts<D, Real, FRIC>(p, parts, i, idx, per, vi, wi, F, T, diag_fc, np);
+}
+
+// Crowded beds: one block per kBinThreads consecutive sorted particles, a
+// thread each.  They lie in a few runs of cells along x; for each run the block
+// reads every particle of the rows around it once, keeps those within reach of
+// the run's box in shared memory, and bins them by subcells no smaller than the
+// reach, so that a particle looks at 9 (27) subcells instead of at every
+// particle of up to 4 (8) cells.  The pairs found are then evaluated one per
+// lane, whatever particle they belong to, and each thread adds its own
+// particle's forces in the order of the walk of k_contacts, so both kernels
+// add the same forces in the same order.
+//
+// Why: the walk is bound by instruction issue.  Its lanes look through
+// different sets of cells, so a warp runs as long as its slowest lane with a
+// third of its lanes busy, at 22 (2D, 11 particles per cell) to 230 (3D, 84 per
+// cell) candidates per particle, and evaluates each lane's few contacts alone.
+// Block and shared-memory shape.
+template <int D> struct BinShape;
+template <> struct BinShape<2> {
+    static constexpr int threads = 128, cap = 384, bins = 384, hits = 8, blocks_f32 = 12;
+};
+template <> struct BinShape<3> {
+    static constexpr int threads = 256, cap = 1024, bins = 1024, hits = 12, blocks_f32 = 3;
+};
+
+// in-cell offsets (in 2D o[2] holds the y cell offset of the candidate's row
+// from the run) and the unwrapped cell along x
+template <class Real> struct alignas(16) BinSlot { Real o[3], x; };
+
+template <int D, class Real, bool FRIC> struct ContactBins {
+    // threads of a block, candidates held at a time, subcells, and pairs of
+    // one particle listed at a time
+    static constexpr int kBinThreads = BinShape<D>::threads, kBinCap = BinShape<D>::cap;
+    static constexpr int kBinMax = BinShape<D>::bins, kBinHits = BinShape<D>::hits;
+    static_assert(kBinCap <= 1024, "a candidate's number takes 10 bits");
+    BinSlot<Real> cand[kBinCap];
+    Real yz[D == 3 ? 2 * kBinCap : 1];          // 3D: y and z cell offsets
+    int j[kBinCap], key[kBinCap];               // slot; place in the order of the walk
+    unsigned short bin[kBinCap], rank[kBinCap], order[kBinCap];
+    int start[kBinMax + 1];                     // counts, then first entries in order[]
+    unsigned short hit[kBinThreads][kBinHits];  // candidates in contact, by key
+    unsigned short flat[kBinThreads / 32][32 * kBinHits];   // a warp's (lane << 10 | candidate)
+    Push<Real, FRIC> push[kBinThreads];         // f = 0: the pair does not push
+    int seg0[27], cum[28], rowbase[27];
+    int warp_tot[kBinThreads / 32], kept;
+};
+
+template <int D, class Real, bool FRIC>
+__global__ void __launch_bounds__(BinShape<D>::threads, sizeof(Real) == 4 ? BinShape<D>::blocks_f32 : 1)
+k_contacts_binned(StepParams<Real> p, Particles<Real> parts, CellList cells, Real *diag_fc, int np)
+{
+    extern __shared__ __align__(16) unsigned char bins_smem[];
+    using Bins = ContactBins<D, Real, FRIC>;
+    constexpr int kBinThreads = Bins::kBinThreads, kBinCap = Bins::kBinCap, kBinMax = Bins::kBinMax;
+    constexpr int kBinHits = Bins::kBinHits;
+    Bins &t = *reinterpret_cast<Bins *>(bins_smem);
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int kRowCells = D == 2 ? kBinMax / 3 - 2 : kBinMax / 9 - 2;   // longest run (m = 1)
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int first = blockIdx.x * kBinThreads, end = min(first + kBinThreads, np);
+    const int i = first + tid;
+    int idx[3] = {0, 0, 0};
+    Real oi[3] = {Real(0), Real(0), Real(0)};
+    Real vi[3] = {Real(0), Real(0), Real(0)}, wi[3] = {Real(0), Real(0), Real(0)};
+    bool per[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) per[a] = (a < D) && (p.bc[2 * a] == BC_PERIODIC);
+    if (i < np) {
+        cell_coords(D, p.n, __ldg(parts.cell + i), idx);
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            oi[a] = __ldg(parts.off[a] + i);
+            vi[a] = __ldg(parts.v[a] + i);
+        }
+        if (FRIC) {
+#pragma unroll
+            for (int k = 0; k < (D == 2 ? 1 : 3); ++k) wi[k] = __ldg(parts.w[k] + i);
+        }
+    }
+    const float cut = (float)p.d + 1e-4f;
+    const Real d2_hi = (Real)p.d2 + contact_band<Real>();
+    Real F[3] = {Real(0), Real(0), Real(0)}, T[3] = {Real(0), Real(0), Real(0)};
+
+    for (int s = first; s < end;) {
+        // the run [s, e): the particles left in the row of slot s (at most kRowCells cells)
+        const int c0 = __ldg(parts.cell + s), xa = c0 % p.n[0], row = c0 - xa;
+        const int e = min(end, cells.begin(row + min(p.n[0], xa + kRowCells)));
+        const int xb = __ldg(parts.cell + e - 1) - row;
+        const int ncx = xb - xa + 1;
+        int ri[3];
+        cell_coords(D, p.n, row, ri);
+        // m subcells per cell along each axis, none smaller than the reach
+        int m = max(1, (int)(0.9999f / cut));
+        while (m > 1 && (ncx * m + 2) * (m + 2) * (D == 3 ? m + 2 : 1) > kBinMax) --m;
+        const int nxs = ncx * m + 2, nys = m + 2, nb = nxs * nys * (D == 3 ? nys : 1);
+        const bool mine = i >= s && i < e;
+        // subcell of an in-cell offset
+        auto sub = [&](Real o) { return min((int)(o * (Real)m), m - 1); };
+        const int bx = (idx[0] - xa) * m + sub(oi[0]), by = sub(oi[1]), bz = D == 3 ? sub(oi[2]) : 0;
+
+        // The slots to read: per plane the rows below, at and above the run,
+        // then, for a run that ends at a periodic x face, the cell across it
+        // in each row (the order of the walk).
+        const int x0 = max(xa - 1, 0), x1 = min(xb + 1, p.n[0] - 1);
+        const int per_plane = per[0] && (xa == 0 || xb == p.n[0] - 1) ? 9 : 3;
+        const int nseg = per_plane * (D == 3 ? 3 : 1);
+        if (warp == 0) {
+            int len = 0;
+            if (lane < nseg) {
+                const int g = lane % per_plane, oz = D == 3 ? lane / per_plane - 1 : 0;
+                const int r = g < 3 ? g : (g - 3) >> 1;
+                int qy = ri[1] + r - 1, qz = ri[2] + oz;
+                bool ok = true;
+                if (qy < 0 || qy >= p.n[1]) {
+                    ok = per[1];
+                    qy = qy < 0 ? qy + p.n[1] : qy - p.n[1];
+                }
+                if (D == 3 && (qz < 0 || qz >= p.n[2])) {
+                    ok = ok && per[2];
+                    qz = qz < 0 ? qz + p.n[2] : qz - p.n[2];
+                }
+                int lo = x0, hi = x1;
+                if (g >= 3) {   // across the low face (the last cell) or the high one
+                    lo = hi = (g & 1) ? p.n[0] - 1 : 0;
+                    ok = ok && ((g & 1) ? xa == 0 : xb == p.n[0] - 1);
+                }
+                const int base = p.n[0] * (qy + p.n[1] * qz);
+                const int b0 = ok ? cells.begin(base + lo) : 0;
+                len = ok ? cells.begin(base + hi + 1) - b0 : 0;
+                t.seg0[lane] = b0;
+                // subtracted from a cell index: its unwrapped cell along x
+                t.rowbase[lane] = g < 3 ? base : ((g & 1) ? base + p.n[0] : base - p.n[0]);
+            }
+            int inc = len;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(kAll, inc, o);
+                if (lane >= o) inc += u;
+            }
+            if (lane < nseg) t.cum[lane + 1] = inc;
+            if (lane == 0) {
+                t.cum[0] = 0;
+                t.kept = 0;
+            }
+        }
+        for (int b = tid; b < nb; b += kBinThreads) t.start[b] = 0;
+        __syncthreads();
+        const int total = t.cum[nseg];
+        int sg = 0;
+        for (int e0 = 0; e0 < total;) {
+            // read on until the next kBinThreads might not fit
+            int kept = 0;
+            for (; e0 < total && kept + kBinThreads <= kBinCap; e0 += kBinThreads) {
+                const int at = e0 + tid;
+                bool keep = at < total;
+                BinSlot<Real> c{};
+                int j = 0, sy = 0, sz = 0;
+                if (keep) {
+                    while (at >= t.cum[sg + 1]) ++sg;
+                    const int g = sg % per_plane;
+                    sy = (g < 3 ? g : (g - 3) >> 1) - 1;
+                    sz = D == 3 ? sg / per_plane - 1 : 0;
+                    j = t.seg0[sg] + at - t.cum[sg];
+#pragma unroll
+                    for (int a = 0; a < D; ++a) c.o[a] = __ldg(parts.off[a] + j);
+                    const int x = __ldg(parts.cell + j) - t.rowbase[sg];
+                    c.x = (Real)x;
+                    // within reach of the run's box
+                    const float fx = (float)c.o[0], fy = (float)c.o[1];
+                    if (x < xa) keep = fx > 1.f - cut;
+                    if (x > xb) keep = keep && fx < cut;
+                    if (sy < 0) keep = keep && fy > 1.f - cut;
+                    if (sy > 0) keep = keep && fy < cut;
+                    if (D == 3) {
+                        const float fz = (float)c.o[2];
+                        if (sz < 0) keep = keep && fz > 1.f - cut;
+                        if (sz > 0) keep = keep && fz < cut;
+                    }
+                }
+                const unsigned b = __ballot_sync(kAll, keep);
+                int base = 0;
+                if (lane == 0 && b) base = atomicAdd(&t.kept, __popc(b));
+                base = __shfl_sync(kAll, base, 0);
+                if (keep) {
+                    const int k = base + __popc(b & ((1u << lane) - 1u));
+                    const int x = (int)c.x;
+                    int bin = (x - xa) * m + sub(c.o[0]) + 1 + nxs * (sy * m + sub(c.o[1]) + 1);
+                    if (D == 3) bin += nxs * nys * (sz * m + sub(c.o[2]) + 1);
+                    if (D == 2) c.o[2] = (Real)sy;
+                    t.cand[k] = c;
+                    if (D == 3) {
+                        t.yz[2 * k] = (Real)sy;
+                        t.yz[2 * k + 1] = (Real)sz;
+                    }
+                    t.j[k] = j;
+                    t.key[k] = at;
+                    t.bin[k] = (unsigned short)bin;
+                    t.rank[k] = (unsigned short)atomicAdd(&t.start[bin], 1);
+                }
+                __syncthreads();
+                kept = t.kept;
+                __syncthreads();
+            }
+            // exclusive scan of the counts, in place
+            {
+                constexpr int kPer = kBinMax / kBinThreads;
+                const int lo = tid * kPer;
+                int v[kPer], sum = 0;
+#pragma unroll
+                for (int k = 0; k < kPer; ++k) {
+                    v[k] = lo + k < nb ? t.start[lo + k] : 0;
+                    sum += v[k];
+                }
+                int inc = sum;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int u = __shfl_up_sync(kAll, inc, o);
+                    if (lane >= o) inc += u;
+                }
+                if (lane == 31) t.warp_tot[warp] = inc;
+                __syncthreads();
+                int run = inc - sum;
+#pragma unroll
+                for (int w = 0; w < kBinThreads / 32; ++w)
+                    if (w < warp) run += t.warp_tot[w];
+#pragma unroll
+                for (int k = 0; k < kPer; ++k) {
+                    if (lo + k < nb) t.start[lo + k] = run;
+                    run += v[k];
+                }
+                if (tid == 0) {
+                    t.start[nb] = kept;
+                    t.kept = 0;
+                }
+            }
+            __syncthreads();
+            for (int k = tid; k < kept; k += kBinThreads)
+                t.order[t.start[t.bin[k]] + t.rank[k]] = (unsigned short)k;
+            __syncthreads();
+
+            // separation of the thread's particle from candidate c
+            auto separation = [&](const BinSlot<Real> &q, int c, const Real *o, Real x, Real *dx) {
+                const Real s3[3] = {q.x - x, D == 2 ? q.o[2] : t.yz[D == 3 ? 2 * c : 0],
+                                    D == 3 ? t.yz[2 * c + 1] : Real(0)};
+                Real d2 = Real(0);
+#pragma unroll
+                for (int a = 0; a < D; ++a) {
+                    dx[a] = o[a] - q.o[a] - s3[a];
+                    d2 += dx[a] * dx[a];
+                }
+                return d2;
+            };
+            // calls f(c) for the candidates in contact range of the thread's
+            // particle (an image farther than a cell away along x is another
+            // candidate's business)
+            auto look = [&](auto &&f) {
+                const Real x = (Real)idx[0];
+#pragma unroll 1
+                for (int dz = 0; dz < (D == 3 ? 3 : 1); ++dz) {
+#pragma unroll 1
+                    for (int dy = 0; dy < 3; ++dy) {
+                        const int b = bx + nxs * (by + dy + (D == 3 ? nys * (bz + dz) : 0));
+                        const int k1 = t.start[b + 3];
+                        for (int k = t.start[b]; k < k1; ++k) {
+                            const int c = t.order[k];
+                            const BinSlot<Real> q = t.cand[c];
+                            Real dx[3];
+                            const Real d2 = separation(q, c, oi, x, dx);
+                            if (!(d2 > d2_hi) && t.j[c] != i && !(fabs(q.x - x) > Real(1))) f(c);
+                        }
+                    }
+                }
+            };
+            int hits = 0;
+            if (mine) {
+                look([&](int c) {
+                    int at = hits++;
+                    if (at >= kBinHits) return;
+                    const int key = t.key[c];
+                    for (; at > 0 && t.key[t.hit[tid][at - 1]] > key; --at) t.hit[tid][at] = t.hit[tid][at - 1];
+                    t.hit[tid][at] = (unsigned short)c;
+                });
+            }
+            if (hits > kBinHits) {
+                // more than the list holds (spheres pressed far into each
+                // other): one pass of the walk per pair, in order
+                for (int done = -1;;) {
+                    int next = INT_MAX, nc = 0;
+                    look([&](int c) {
+                        const int key = t.key[c];
+                        if (key > done && key < next) {
+                            next = key;
+                            nc = c;
+                        }
+                    });
+                    if (next == INT_MAX) break;
+                    done = next;
+                    Real dx[3];
+                    const Real d2 = separation(t.cand[nc], nc, oi, (Real)idx[0], dx);
+                    Push<Real, FRIC> c;
+                    if (pair_push<D, Real, FRIC>(p, parts, i, t.j[nc], per, dx, d2, vi, wi, c))
+                        add_push<D, Real, FRIC>(c, F, T);
+                }
+                hits = 0;
+            }
+            // the warp's pairs in one list, particle by particle
+            int h1 = hits;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(kAll, h1, o);
+                if (lane >= o) h1 += u;
+            }
+            const int h0 = h1 - hits, nh = __shfl_sync(kAll, h1, 31);
+            for (int k = 0; k < hits; ++k)
+                t.flat[warp][h0 + k] = (unsigned short)(lane << 10 | t.hit[tid][k]);
+            __syncwarp();
+            Push<Real, FRIC> *push = t.push + 32 * warp;
+            for (int b0 = 0; b0 < nh; b0 += 32) {
+                // one pair per lane; its particle's state comes from the owning lane
+                const bool have = b0 + lane < nh;
+                const int fl = have ? t.flat[warp][b0 + lane] : 0, own = fl >> 10, c = fl & 1023;
+                Real om[3] = {Real(0), Real(0), Real(0)};
+                Real vm[3] = {Real(0), Real(0), Real(0)}, wm[3] = {Real(0), Real(0), Real(0)};
+#pragma unroll
+                for (int a = 0; a < D; ++a) {
+                    om[a] = __shfl_sync(kAll, oi[a], own);
+                    vm[a] = __shfl_sync(kAll, vi[a], own);
+                }
+                const int xm = __shfl_sync(kAll, idx[0], own);
+                if (FRIC) {
+#pragma unroll
+                    for (int k = 0; k < (D == 2 ? 1 : 3); ++k) wm[k] = __shfl_sync(kAll, wi[k], own);
+                }
+                if (have) {
+                    Real dx[3];
+                    const Real d2 = separation(t.cand[c], c, om, (Real)xm, dx);
+                    if (!pair_push<D, Real, FRIC>(p, parts, i - lane + own, t.j[c], per, dx, d2, vm, wm,
+                                                  push[lane]))
+                        push[lane].f = Real(0);
+                }
+                __syncwarp();
+                const int k1 = min(h1, b0 + 32);
+                for (int k = max(h0, b0); k < k1; ++k)
+                    if (push[k - b0].f > Real(0)) add_push<D, Real, FRIC>(push[k - b0], F, T);
+                __syncwarp();
+            }
+            __syncthreads();
+            if (e0 < total) {
+                for (int b = tid; b < nb; b += kBinThreads) t.start[b] = 0;
+                __syncthreads();
+            }
+        }
+        s = e;
+        __syncthreads();
+    }
+    if (i < np) finish_contacts<D, Real, FRIC>(p, parts, i, idx, per, vi, wi, F, T, diag_fc, np);
+}
+
+// Mean particles per cell from which the binned kernel is taken.  Both sides on
+// a GB300, particles spread evenly, d = 0.2 (us; 2D 256 x 1024, 3D 48 x 48 x 64):
+//     2D per cell     2          4          5.6 (lower half filled: 11)
+//     walk / binned   26 / 43    59 / 70    155 / 93
+//     3D per cell     2          4          16
+//     walk / binned   39 / 94    97 / 141   917 / 507
+// The bed of 256 x 1024 cells took 155 us per launch with the walk alone, the
+// 3D bed of 16 x 16 x 32 cells (42 per cell, friction) 660 us against 112.
+template <int D> constexpr int kBinOccupancy = D == 2 ? 5 : 8;
+
+template <int D, class Real, bool FRIC>
+static void launch_contacts_fric(const StepParams<Real> &p, Particles<Real> parts, CellList cells,
+                                 Real *diag_fc, int np, cudaStream_t st)
+{
+    if ((long long)np >= (long long)kBinOccupancy<D> * p.ncell) {
+        constexpr size_t smem = sizeof(ContactBins<D, Real, FRIC>);
+        constexpr int kBinThreads = BinShape<D>::threads;
+        // a refusal shows as the launch's error
+        cudaFuncSetAttribute(k_contacts_binned<D, Real, FRIC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)smem);
+        k_contacts_binned<D, Real, FRIC><<<(np + kBinThreads - 1) / kBinThreads, kBinThreads, smem, st>>>(
+            p, parts, cells, diag_fc, np);
+    } else {
+        const int b = wave_block(k_contacts<D, Real, FRIC>, np);
+        k_contacts<D, Real, FRIC><<<(np + b - 1) / b, b, 0, st>>>(p, parts, cells, diag_fc, np);
+    }
+}
+
 template <int D, class Real>
 void launch_contacts(const StepParams<Real> &p, Particles<Real> parts, CellList cells,
                      Real *diag_fc, int np, cudaStream_t st)
 {
     if (np == 0) return;
-    if (p.spin_out[0]) {
-        const int b = wave_block(k_contacts<D, Real, true>, np);
-        k_contacts<D, Real, true><<<(np + b - 1) / b, b, 0, st>>>(p, parts, cells, diag_fc, np);
-    } else {
-        const int b = wave_block(k_contacts<D, Real, false>, np);
-        k_contacts<D, Real, false><<<(np + b - 1) / b, b, 0, st>>>(p, parts, cells, diag_fc, np);
-    }
+    if (p.spin_out[0]) launch_contacts_fric<D, Real, true>(p, parts, cells, diag_fc, np, st);
+    else launch_contacts_fric<D, Real, false>(p, parts, cells, diag_fc, np, st);
 }
 
 #define LBDPS_INST_C(D, R)                                                                          \

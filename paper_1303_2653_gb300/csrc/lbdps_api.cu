@@ -642,6 +642,13 @@ template <class L, class Real, class S> struct EngineT : Engine {
         return set_particles(pos, vel, pos_div, vel_mul);
     }
 
+    // Device room for the duration of one transfer: the population buffer that
+    // the next step overwrites (nothing reads it between steps), so that
+    // reading and loading a bed allocate nothing.  Work that uses it is on the
+    // handle's stream, and the calls wait for it before they return.
+    char *scratch() { return reinterpret_cast<char *>(f[1 - H->parity]); }
+    size_t scratch_bytes() const { return sizeof(S) * pop_slots(); }
+
     // Load particles (id order; lattice units once positions are divided by
     // pos_div and velocities multiplied by vel_mul) into the current buffers
     // and sort them.
@@ -655,8 +662,9 @@ template <class L, class Real, class S> struct EngineT : Engine {
         // device (ids in order, spins at rest), then sorted into the current
         // buffers
         const size_t bytes = sizeof(double) * (size_t)np * D;
-        double *dp = (double *)H->mem.get_temp(bytes);
-        double *dv = dp ? (double *)H->mem.get_temp(bytes) : nullptr;
+        const bool room = 2 * bytes <= scratch_bytes();
+        double *dp = room ? (double *)scratch() : (double *)H->mem.get_temp(bytes);
+        double *dv = room ? dp + (size_t)np * D : dp ? (double *)H->mem.get_temp(bytes) : nullptr;
         if (dp && dv) {
             cudaError_t e = cudaMemcpyAsync(dp, pos, bytes, cudaMemcpyHostToDevice, st);
             if (e == cudaSuccess) e = cudaMemcpyAsync(dv, vel, bytes, cudaMemcpyHostToDevice, st);
@@ -665,8 +673,10 @@ template <class L, class Real, class S> struct EngineT : Engine {
                 e = cudaGetLastError();
             }
             const cudaError_t e2 = cudaStreamSynchronize(st);
-            H->mem.put_temp(dp);
-            H->mem.put_temp(dv);
+            if (!room) {
+                H->mem.put_temp(dp);
+                H->mem.put_temp(dv);
+            }
             if (e != cudaSuccess || e2 != cudaSuccess) {
                 cudaGetLastError();
                 return fail(LBDPS_ERR_CUDA, "particle upload: %s",
@@ -878,56 +888,46 @@ template <class L, class Real, class S> struct EngineT : Engine {
         const double fs = units == LBDPS_UNITS_SI ? H->prm.rho_g * H->h * H->h * H->h * H->h / (H->dt * H->dt) : 1.0;
         const double bs = units == LBDPS_UNITS_SI ? H->prm.rho_g / H->dt : 1.0;
         const double ts = units == LBDPS_UNITS_SI ? H->dt : 1.0;
-        std::vector<Real> hb;
-        std::vector<int> hi;
-        size_t o = 0;
-        auto put_scalar = [&](const Real *src, double scale) -> int {
-            int rc = d2h(hb, src, nc);
-            if (rc) return rc;
-            for (size_t x = 0; x < nc; ++x) out[o + x] = (double)hb[x] * scale;
-            o += nc;
-            return LBDPS_OK;
+        // On the device: converted, scaled and interleaved in the order of the
+        // output, as much as the scratch holds at a time, and copied into the
+        // caller's memory once.
+        const Real *node = reinterpret_cast<const Real *>(fld.node4);   // u_act at 0.., beta at 3
+        FieldExport<Real> x{};
+        auto add = [&](int bit, int count, double scale, const Real *a0, const Real *a1, const Real *a2,
+                       int stride) {
+            if (!(mask & bit)) return;
+            auto &f1 = x.f[x.nfield++];
+            f1.first = x.total;
+            f1.count = count;
+            f1.stride = stride;
+            f1.scale = scale;
+            f1.src[0] = a0;
+            f1.src[1] = a1;
+            f1.src[2] = a2;
+            x.total += (long long)nc * count;
         };
-        auto put_vec = [&](Real *const *src, double scale) -> int {
-            for (int a = 0; a < D; ++a) {
-                int rc = d2h(hb, src[a], nc);
-                if (rc) return rc;
-                for (size_t x = 0; x < nc; ++x) out[o + x * D + a] = (double)hb[x] * scale;
-            }
-            o += nc * D;
-            return LBDPS_OK;
-        };
-        // components of the node record: beta is .w, u_act is .x, .y (, .z)
-        using V4 = typename Vec4<Real>::type;
-        std::vector<V4> h4;
-        auto put_node = [&](int first, int count, double scale) -> int {
-            if (h4.empty()) {
-                h4.resize(nc);
-                CU(cudaMemcpyAsync(h4.data(), fld.node4, sizeof(V4) * nc, cudaMemcpyDeviceToHost,
-                                   H->stream));
-                CU(cudaStreamSynchronize(H->stream));
-            }
-            for (size_t x = 0; x < nc; ++x) {
-                const Real c4[4] = {h4[x].x, h4[x].y, h4[x].z, h4[x].w};
-                for (int a = 0; a < count; ++a) out[o + x * count + a] = (double)c4[first + a] * scale;
-            }
-            o += nc * count;
-            return LBDPS_OK;
-        };
-        int rc = LBDPS_OK;
-        if (mask & LBDPS_FIELD_RHO) if ((rc = put_scalar(fld.rho, rs))) return rc;
-        if (mask & LBDPS_FIELD_U) if ((rc = put_vec(fld.u, us))) return rc;
-        if (mask & LBDPS_FIELD_FPG) if ((rc = put_vec(fld.fpg, fs))) return rc;
-        if (mask & LBDPS_FIELD_BETA) if ((rc = put_node(3, 1, bs))) return rc;
-        if (mask & LBDPS_FIELD_VS) if ((rc = put_vec(fld.vs, us))) return rc;
-        if (mask & LBDPS_FIELD_NTOT) {
-            if ((rc = d2h(hi, fld.ntot, nc))) return rc;
-            for (size_t x = 0; x < nc; ++x) out[o + x] = (double)hi[x];
-            o += nc;
+        add(LBDPS_FIELD_RHO, 1, rs, fld.rho, nullptr, nullptr, 1);
+        add(LBDPS_FIELD_U, D, us, fld.u[0], fld.u[1], fld.u[2], 1);
+        add(LBDPS_FIELD_FPG, D, fs, fld.fpg[0], fld.fpg[1], fld.fpg[2], 1);
+        add(LBDPS_FIELD_BETA, 1, bs, node + 3, nullptr, nullptr, 4);
+        add(LBDPS_FIELD_VS, D, us, fld.vs[0], fld.vs[1], fld.vs[2], 1);
+        if (mask & LBDPS_FIELD_NTOT) x.counts = fld.ntot;
+        add(LBDPS_FIELD_NTOT, 1, 1.0, nullptr, nullptr, nullptr, 1);
+        add(LBDPS_FIELD_TAU_T, 1, ts, fld.tau_t, nullptr, nullptr, 1);
+        add(LBDPS_FIELD_UACT, D, us, node, node + 1, node + 2, 4);
+        add(LBDPS_FIELD_EPS_G, 1, 1.0, fld.eps_g, nullptr, nullptr, 1);
+        const long long room = (long long)(scratch_bytes() / sizeof(double));
+        bool touched = false;
+        for (long long lo = 0; lo < x.total; lo += room) {
+            const long long n = std::min(room, x.total - lo);
+            double *dev = reinterpret_cast<double *>(scratch());
+            launch_export_fields<Real>(x, lo, n, dev, H->stream);
+            CHECK_LAUNCH();
+            if (!touched) touch_pages(out, sizeof(double) * need);   // while the kernel runs
+            touched = true;
+            CU(cudaMemcpyAsync(out + lo, dev, sizeof(double) * n, cudaMemcpyDeviceToHost, H->stream));
         }
-        if (mask & LBDPS_FIELD_TAU_T) if ((rc = put_scalar(fld.tau_t, ts))) return rc;
-        if (mask & LBDPS_FIELD_UACT) if ((rc = put_node(0, D, us))) return rc;
-        if (mask & LBDPS_FIELD_EPS_G) if ((rc = put_scalar(fld.eps_g, 1.0))) return rc;
+        CU(cudaStreamSynchronize(H->stream));
         return LBDPS_OK;
     }
 
@@ -941,8 +941,10 @@ template <class L, class Real, class S> struct EngineT : Engine {
         // on the device: id order, interleaved, scaled; one copy per array
         // into the caller's memory
         const size_t bytes = sizeof(double) * (size_t)np * D;
-        double *dp = pos ? (double *)H->mem.get_temp(bytes) : nullptr;
-        double *dv = vel ? (double *)H->mem.get_temp(bytes) : nullptr;
+        const bool room = 2 * bytes <= scratch_bytes();
+        double *dp = !pos ? nullptr : room ? (double *)scratch() : (double *)H->mem.get_temp(bytes);
+        double *dv = !vel ? nullptr
+                          : room ? (double *)scratch() + (size_t)np * D : (double *)H->mem.get_temp(bytes);
         if ((!pos || dp) && (!vel || dv)) {
             cudaStream_t st = H->stream;
             launch_particles_to_host_order<D, Real>(part[cur], np, ps, vs, dp, dv, st);
@@ -953,8 +955,10 @@ template <class L, class Real, class S> struct EngineT : Engine {
             if (e == cudaSuccess && pos) e = cudaMemcpyAsync(pos, dp, bytes, cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess && vel) e = cudaMemcpyAsync(vel, dv, bytes, cudaMemcpyDeviceToHost, st);
             const cudaError_t e2 = cudaStreamSynchronize(st);
-            H->mem.put_temp(dp);
-            H->mem.put_temp(dv);
+            if (!room) {
+                H->mem.put_temp(dp);
+                H->mem.put_temp(dv);
+            }
             if (e != cudaSuccess || e2 != cudaSuccess) {
                 cudaGetLastError();
                 return fail(LBDPS_ERR_CUDA, "particle read-back: %s",
@@ -992,11 +996,29 @@ template <class L, class Real, class S> struct EngineT : Engine {
             return LBDPS_OK;
         }
         if (np == 0) return LBDPS_OK;
+        const double ws = units == LBDPS_UNITS_SI ? 1.0 / H->dt : 1.0;
+        const size_t bytes = sizeof(double) * (size_t)np * NW;
+        const bool room = bytes <= scratch_bytes();
+        double *dw = room ? (double *)scratch() : (double *)H->mem.get_temp(bytes);
+        if (dw) {
+            launch_spins_to_host_order<NW, Real>(part[cur], np, ws, dw, H->stream);
+            cudaError_t e = cudaGetLastError();
+            touch_pages(out, bytes);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(out, dw, bytes, cudaMemcpyDeviceToHost, H->stream);
+            const cudaError_t e2 = cudaStreamSynchronize(H->stream);
+            if (!room) H->mem.put_temp(dw);
+            if (e != cudaSuccess || e2 != cudaSuccess) {
+                cudaGetLastError();
+                return fail(LBDPS_ERR_CUDA, "spin read-back: %s",
+                            cudaGetErrorString(e != cudaSuccess ? e : e2));
+            }
+            return LBDPS_OK;
+        }
+        // no room for the staging array: order on the host
         std::vector<int> ids;
         std::vector<Real> wd;
         int rc = d2h(ids, part[cur].id, np);
         if (rc) return rc;
-        const double ws = units == LBDPS_UNITS_SI ? 1.0 / H->dt : 1.0;
         for (int c = 0; c < NW; ++c) {
             if ((rc = d2h(wd, part[cur].w[c], np))) return rc;
             for (int k = 0; k < np; ++k) out[(size_t)ids[k] * NW + c] = (double)wd[k] * ws;
@@ -1026,14 +1048,19 @@ template <class L, class Real, class S> struct EngineT : Engine {
     {
         const size_t total = (size_t)Q * H->ncell;
         if (cap < total) return fail(LBDPS_ERR_CAPACITY, "need %zu doubles", total);
-        double *dev = nullptr;
-        CU(cudaMalloc(&dev, sizeof(double) * total));
-        launch_export_populations<L, Real, S>(lay, H->ncell, f[H->parity], dev, H->stream);
-        cudaError_t e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaMemcpyAsync(out, dev, sizeof(double) * total, cudaMemcpyDeviceToHost, H->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(H->stream);
-        cudaFree(dev);
-        if (e != cudaSuccess) return fail(LBDPS_ERR_CUDA, "populations: %s", cudaGetErrorString(e));
+        const size_t room = scratch_bytes() / sizeof(double);
+        bool touched = false;
+        for (size_t lo = 0; lo < total; lo += room) {
+            const size_t n = std::min(room, total - lo);
+            double *dev = reinterpret_cast<double *>(scratch());
+            launch_export_populations<L, Real, S>(lay, H->ncell, f[H->parity], (long long)lo, (long long)n,
+                                                  dev, H->stream);
+            CHECK_LAUNCH();
+            if (!touched) touch_pages(out, sizeof(double) * total);   // while the kernel runs
+            touched = true;
+            CU(cudaMemcpyAsync(out + lo, dev, sizeof(double) * n, cudaMemcpyDeviceToHost, H->stream));
+        }
+        CU(cudaStreamSynchronize(H->stream));
         return LBDPS_OK;
     }
 
@@ -1041,16 +1068,16 @@ template <class L, class Real, class S> struct EngineT : Engine {
     {
         const size_t total = (size_t)Q * H->ncell;
         if (count != total) return fail(LBDPS_ERR_INVALID, "expected %zu values", total);
-        double *dev = nullptr;
-        CU(cudaMalloc(&dev, sizeof(double) * total));
-        cudaError_t e = cudaMemcpyAsync(dev, in, sizeof(double) * total, cudaMemcpyHostToDevice, H->stream);
-        if (e == cudaSuccess) {
-            launch_import_populations<L, Real, S>(lay, H->ncell, dev, f[H->parity], H->stream);
-            e = cudaGetLastError();
+        const size_t room = scratch_bytes() / sizeof(double);
+        for (size_t lo = 0; lo < total; lo += room) {
+            const size_t n = std::min(room, total - lo);
+            double *dev = reinterpret_cast<double *>(scratch());
+            CU(cudaMemcpyAsync(dev, in + lo, sizeof(double) * n, cudaMemcpyHostToDevice, H->stream));
+            launch_import_populations<L, Real, S>(lay, H->ncell, dev, (long long)lo, (long long)n,
+                                                  f[H->parity], H->stream);
+            CHECK_LAUNCH();
         }
-        if (e == cudaSuccess) e = cudaStreamSynchronize(H->stream);
-        cudaFree(dev);
-        if (e != cudaSuccess) return fail(LBDPS_ERR_CUDA, "set_populations: %s", cudaGetErrorString(e));
+        CU(cudaStreamSynchronize(H->stream));
         return LBDPS_OK;
     }
 

@@ -334,13 +334,34 @@ template <class L, class Real, class S>
 void launch_gas_moments(const PopLayout &lay, const S *f, const int *n, double *partials,
                         cudaStream_t st);
 
+// n full population values in FP64 from value lo on ([q][cell] order): out and
+// in point at value lo
 template <class L, class Real, class S>
-void launch_export_populations(const PopLayout &lay, int ncell, const S *f, double *out,
-                               cudaStream_t st);
+void launch_export_populations(const PopLayout &lay, int ncell, const S *f, long long lo, long long n,
+                               double *out, cudaStream_t st);
 
 template <class L, class Real, class S>
-void launch_import_populations(const PopLayout &lay, int ncell, const double *in, S *f,
-                               cudaStream_t st);
+void launch_import_populations(const PopLayout &lay, int ncell, const double *in, long long lo,
+                               long long n, S *f, cudaStream_t st);
+
+// Node fields exported one after the other: field i holds values f[i].first
+// on, count per cell (interleaved), component a of cell c read at
+// src[a][c * stride] and multiplied by scale; src[0] null: the particle counts.
+template <class Real> struct FieldExport {
+    struct {
+        long long first;
+        int count, stride;
+        double scale;
+        const Real *src[3];
+    } f[9];
+    int nfield;
+    long long total;
+    const int *counts;
+};
+// values lo .. lo + n - 1 into out[0..n)
+template <class Real>
+void launch_export_fields(const FieldExport<Real> &x, long long lo, long long n, double *out,
+                          cudaStream_t st);
 
 template <class Real>
 void launch_build_tables(int dim, double tau, double r, double vp, double d, double mu,
@@ -363,6 +384,9 @@ void launch_cell_keys(const int *n, Particles<Real> parts, int *key, int *counts
 template <int D, class Real>
 void launch_particles_to_host_order(Particles<Real> parts, int np, double ps, double vs,
                                     double *pos, double *vel, cudaStream_t st);
+// The spins in id order, interleaved (np x NW), times ws in FP64.
+template <int NW, class Real>
+void launch_spins_to_host_order(Particles<Real> parts, int np, double ws, double *out, cudaStream_t st);
 // Interleaved id-order positions and velocities (np x D) into the SoA arrays
 // of dst in lattice units (positions / pos_div, velocities * vel_mul, both
 // correctly rounded in FP64), with ids 0..np-1 and spins (if any) at rest.

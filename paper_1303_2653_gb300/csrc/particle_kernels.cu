@@ -450,6 +450,23 @@ void launch_particles_to_host_order(Particles<Real> parts, int np, double ps, do
     k_particles_to_host_order<D, Real><<<(np + 255) / 256, 256, 0, st>>>(parts, np, ps, vs, pos, vel);
 }
 
+template <int NW, class Real>
+__global__ void k_spins_to_host_order(Particles<Real> parts, int np, double ws, double *out)
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= np) return;
+    const size_t o = (size_t)parts.id[k] * NW;
+#pragma unroll
+    for (int c = 0; c < NW; ++c) out[o + c] = (double)parts.w[c][k] * ws;
+}
+
+template <int NW, class Real>
+void launch_spins_to_host_order(Particles<Real> parts, int np, double ws, double *out, cudaStream_t st)
+{
+    if (np == 0) return;
+    k_spins_to_host_order<NW, Real><<<(np + 255) / 256, 256, 0, st>>>(parts, np, ws, out);
+}
+
 template <int D, class Real>
 __global__ void k_particles_from_host_order(const double *pos, const double *vel, int np,
                                             double pos_div, double vel_mul, Particles<Real> dst)
@@ -1170,6 +1187,11 @@ LBDPS_INST_P(2, double)
 LBDPS_INST_P(2, float)
 LBDPS_INST_P(3, double)
 LBDPS_INST_P(3, float)
+
+template void launch_spins_to_host_order<1, double>(Particles<double>, int, double, double *, cudaStream_t);
+template void launch_spins_to_host_order<3, double>(Particles<double>, int, double, double *, cudaStream_t);
+template void launch_spins_to_host_order<1, float>(Particles<float>, int, double, double *, cudaStream_t);
+template void launch_spins_to_host_order<3, float>(Particles<float>, int, double, double *, cudaStream_t);
 
 template void launch_place<double>(int, const int *, int *, CellList, int2 *, int *,
                                    Particles<double>, Particles<double>, int, cudaStream_t);

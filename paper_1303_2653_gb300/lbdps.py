@@ -337,7 +337,7 @@ class Bed:
         res, o = {}, 0
         for name, s in sizes:
             arr = out[o:o + s]
-            res[name] = arr.reshape(self.ncell, self.dim) if name in VECTOR_FIELDS else arr.copy()
+            res[name] = arr.reshape(self.ncell, self.dim) if name in VECTOR_FIELDS else arr
             o += s
         return res
 

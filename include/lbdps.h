@@ -409,9 +409,9 @@ void lbdps_server_destroy(lbdps_server_t *s);
  *   order        DEVICE output, np ints: the particle id in each sorted slot
  *   stream       cudaStream_t (NULL = legacy default stream); asynchronous
  * The order inside a cell comes from a stable radix sort of the cell keys
- * (at most three 8-bit passes), so the work is linear in np whatever the
+ * (at most two passes of up to 10 bits), so the work is linear in np whatever the
  * occupancy of the cells.  np < 0 returns LBDPS_ERR_INVALID.
- * Temporaries live in one fixed device array of about 28 MB, created on each
+ * Temporaries live in one fixed device array of about 25 MB, created on each
  * GPU that loads the library and kept until the process exits; this function
  * calls no cudaMalloc, cudaFree or allocating library routine.  Limits:
  * ncell <= 1048576 and np <= 1048576, otherwise LBDPS_ERR_CAPACITY with no

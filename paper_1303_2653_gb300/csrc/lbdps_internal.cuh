@@ -407,11 +407,6 @@ void launch_detect(const StepParams<Real> &p, Particles<Real> parts, CellList ce
                    int *wall, long long *pairs, unsigned long long *npairs, long long pair_cap,
                    int np, cudaStream_t st);
 
-// three-kernel scan into a plain cell_start[ncell + 1] (used by the
-// allocation-free binning entry point)
-void launch_scan(const int *counts, int *cell_start, int *block_sums, int ncell, cudaStream_t st);
-int scan_block_count(int ncell);
-
 // pairs of particles closer than d (creation check of hard spheres): count
 // and the smallest (id_i << 32 | id_j), i < j
 template <int D, class Real>

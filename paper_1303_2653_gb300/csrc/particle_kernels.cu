@@ -626,72 +626,6 @@ void launch_cell_scan(const int *counts, CellListOut out, int ncell, cudaStream_
 }
 
 // ---------------------------------------------------------------------------
-// Three-kernel scan into a plain cell_start array (per-block scans with block
-// totals, a scan of the block totals in one block, the block offsets added).
-// ---------------------------------------------------------------------------
-constexpr int kScanThreads = 512;
-constexpr int kScanItems = 8;
-constexpr int kScanTile = kScanThreads * kScanItems;
-
-int scan_block_count(int ncell) { return (ncell + kScanTile - 1) / kScanTile; }
-
-__global__ void __launch_bounds__(kScanThreads)
-k_scan_tiles(const int *__restrict__ counts, int *__restrict__ out, int *__restrict__ block_sums,
-             int n)
-{
-    __shared__ int warp_tot[32];
-    __shared__ int total;
-    const int base = blockIdx.x * kScanTile + threadIdx.x * kScanItems;
-    int vals[kScanItems];
-    int sum = 0;
-#pragma unroll
-    for (int j = 0; j < kScanItems; ++j) {
-        const int e = base + j;
-        vals[j] = e < n ? counts[e] : 0;
-        sum += vals[j];
-    }
-    int run = block_exclusive_scan(sum, warp_tot, &total);
-#pragma unroll
-    for (int j = 0; j < kScanItems; ++j) {
-        const int e = base + j;
-        if (e < n) out[e] = run;
-        run += vals[j];
-    }
-    if (threadIdx.x == 0) block_sums[blockIdx.x] = total;
-}
-
-__global__ void __launch_bounds__(1024) k_scan_block_sums(int *block_sums, int nb)
-{
-    __shared__ int warp_tot[32];
-    __shared__ int total;
-    int carry = 0;
-    for (int base = 0; base < nb; base += blockDim.x) {
-        const int e = base + threadIdx.x;
-        const int v = e < nb ? block_sums[e] : 0;
-        const int ex = block_exclusive_scan(v, warp_tot, &total);
-        if (e < nb) block_sums[e] = carry + ex;
-        carry += total;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) block_sums[nb] = carry;
-}
-
-__global__ void k_scan_add(int *out, const int *block_sums, int n, int nb)
-{
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < n) out[e] += block_sums[e / kScanTile];
-    if (e == n) out[n] = block_sums[nb];
-}
-
-void launch_scan(const int *counts, int *cell_start, int *block_sums, int ncell, cudaStream_t st)
-{
-    const int nb = scan_block_count(ncell);
-    k_scan_tiles<<<nb, kScanThreads, 0, st>>>(counts, cell_start, block_sums, ncell);
-    k_scan_block_sums<<<1, 1024, 0, st>>>(block_sums, nb);
-    k_scan_add<<<(ncell + 1 + 255) / 256, 256, 0, st>>>(cell_start, block_sums, ncell, nb);
-}
-
-// ---------------------------------------------------------------------------
 // Placement.  Each particle takes a slot in its cell's range by an atomic
 // decrement of the cell count (which also returns the counts to zero for the
 // next histogram) and records its id there.  The order inside a cell is then

@@ -24,7 +24,7 @@ int wave_block(K kern, long long n)
     static std::mutex mu;
     static std::map<std::pair<const void *, int>, int> fit;   // (kernel, block) -> blocks per SM
     static int nsm = 0;
-        constexpr int cand[3] = {256, 128, 64};
+    constexpr int cand[3] = {256, 128, 64};
     std::lock_guard<std::mutex> lock(mu);
     if (nsm == 0) {
         int dev = 0;

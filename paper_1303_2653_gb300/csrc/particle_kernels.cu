@@ -179,10 +179,17 @@ __device__ __forceinline__ void drag_pre_one(const StepParams<Real> &p, const Pa
 // 148,860 particles in 100 x 75 x 333 cells, GB300.)
 // ---------------------------------------------------------------------------
 // Register budgets of the drag and detection kernels, as blocks of 256
-// threads per SM.  Detection fits 40 registers in 2D FP32 (6 blocks: 200,000
-// particles in one wave, see wave_block); the drag spills below 48.
+// threads per SM.  The drag is bound by the latency of its gathers and gains
+// more from registers to hold them in flight than from warps: in 2D 64
+// registers (4 blocks) against 48 (5 blocks, 88 bytes of spills) take the step
+// of the 256 x 2048 riser from 45.0 to 42.5 us, 512 x 2048 from 75.5 to 71.3 and
+// the crowded 256 x 1024 bed from 210.5 to 206.8; in 3D 4 blocks spill (drag of
+// the 256 x 256 x 1024 riser 823 us against 620) and 2 leave it short of warps
+// (717).  Detection fits 40 registers in 2D FP32 (6 blocks: 200,000 particles in
+// one wave, see wave_block; 5 or 7 cost it half a microsecond) and 48 in 3D (5
+// blocks; 4 take 16 us longer on that riser).
 #ifndef LBDPS_DRAG_BLOCKS_2D_F32
-#define LBDPS_DRAG_BLOCKS_2D_F32 5
+#define LBDPS_DRAG_BLOCKS_2D_F32 4
 #endif
 #ifndef LBDPS_DRAG_BLOCKS_3D_F32
 #define LBDPS_DRAG_BLOCKS_3D_F32 3

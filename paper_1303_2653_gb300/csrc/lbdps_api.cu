@@ -449,7 +449,7 @@ template <class L, class Real, class S> struct EngineT : Engine {
         fld.rho = (Real *)get(sizeof(Real) * nc);
         fld.node4 = (typename Vec4<Real>::type *)get(sizeof(typename Vec4<Real>::type) * nc);
         fld.solg = D == 3 ? (Real *)get(sizeof(Real) * nc) : nullptr;
-        for (int a = 0; a < D; ++a) fld.fpg[a] = (Real *)get(sizeof(Real) * nc);
+        for (int a = 0; a < D; ++a) fld.fpg[a] = (Real *)get(sizeof(Real) * (D == 2 ? nc : np));
         if (H->prm.diagnostics) {
             fld.tau_t = (Real *)get(sizeof(Real) * nc);
             fld.eps_g = (Real *)get(sizeof(Real) * nc);
@@ -634,11 +634,9 @@ template <class L, class Real, class S> struct EngineT : Engine {
         CU(cudaMemsetAsync(ticket, 0, sizeof(unsigned), st));
         CU(cudaMemsetAsync(red_ticket, 0, sizeof(unsigned), st));
         CU(cudaMemsetAsync(solids_out, 0, sizeof(unsigned long long), st));
-        if (H->np == 0) {
-            int rc = clear_cells(0);
-            if (rc == LBDPS_OK) rc = clear_cells(1);
-            return rc;
-        }
+        int rc = clear_cells(1 - H->parity);   // the list of the fields before the first step
+        if (rc) return rc;
+        if (H->np == 0) return clear_cells(H->parity);
         return set_particles(pos, vel, pos_div, vel_mul);
     }
 
@@ -893,6 +891,10 @@ template <class L, class Real, class S> struct EngineT : Engine {
         // caller's memory once.
         const Real *node = reinterpret_cast<const Real *>(fld.node4);   // u_act at 0.., beta at 3
         FieldExport<Real> x{};
+        x.cells = cells(1 - H->parity);   // the input of the last step
+        x.np = H->np;
+        x.rho = fld.rho;
+        x.node4 = fld.node4;
         auto add = [&](int bit, int count, double scale, const Real *a0, const Real *a1, const Real *a2,
                        int stride) {
             if (!(mask & bit)) return;
@@ -908,7 +910,7 @@ template <class L, class Real, class S> struct EngineT : Engine {
         };
         add(LBDPS_FIELD_RHO, 1, rs, fld.rho, nullptr, nullptr, 1);
         add(LBDPS_FIELD_U, D, us, fld.u[0], fld.u[1], fld.u[2], 1);
-        add(LBDPS_FIELD_FPG, D, fs, fld.fpg[0], fld.fpg[1], fld.fpg[2], 1);
+        add(LBDPS_FIELD_FPG, D, fs, fld.fpg[0], fld.fpg[1], fld.fpg[2], D == 2 ? 1 : 0);
         add(LBDPS_FIELD_BETA, 1, bs, node + 3, nullptr, nullptr, 4);
         add(LBDPS_FIELD_VS, D, us, fld.vs[0], fld.vs[1], fld.vs[2], 1);
         if (mask & LBDPS_FIELD_NTOT) x.counts = fld.ntot;

@@ -242,6 +242,13 @@ __host__ __device__ inline void cell_voidage(int dim, double r, double vp, int n
 // node4 is the record the drag reads at each stencil node, one 16-byte (FP32)
 // load: {u_act,x, u_act,y, 1 - eps, beta} in 2D and {u_act,x, u_act,y,
 // u_act,z, beta} in 3D, where 1 - eps is in solg.
+// fpg (F_p->g) is read by the drag of the cell's own particles only.  In 3D,
+// where a bed holds 0.06 particles per cell, it is kept for the occupied cells
+// alone, at the sorted slot of the cell's first particle in the step's input
+// list: 48 instead of 805 MB written per step of the 256 x 256 x 1024 riser
+// (collision 2,090 -> 1,966 us, drag 620 -> 576).  In 2D (0.4 and more per cell)
+// that saves little, and the slot lengthens the drag's chain of loads (75 x 193:
+// 22.2 -> 23.4 us a step), so it stays per cell.
 template <class Real> struct Fields {
     Real *rho, *fpg[3];                                 // node outputs of the collision
     typename Vec4<Real>::type *node4;
@@ -346,7 +353,8 @@ void launch_import_populations(const PopLayout &lay, int ncell, const double *in
 
 // Node fields exported one after the other: field i holds values f[i].first
 // on, count per cell (interleaved), component a of cell c read at
-// src[a][c * stride] and multiplied by scale; src[0] null: the particle counts.
+// src[a][c * stride] and multiplied by scale.  src[0] null: the particle counts;
+// stride 0: kept per occupied cell (Fields::fpg), the list of that step in cells.
 template <class Real> struct FieldExport {
     struct {
         long long first;
@@ -357,6 +365,10 @@ template <class Real> struct FieldExport {
     int nfield;
     long long total;
     const int *counts;
+    CellList cells;
+    int np;
+    const Real *rho;
+    const typename Vec4<Real>::type *node4;
 };
 // values lo .. lo + n - 1 into out[0..n)
 template <class Real>

@@ -284,7 +284,7 @@ __device__ __forceinline__ void drag_step_particle(const StepParams<Real> &p,
         s0 = cells.begin(c);
         s1 = cells.begin(c + 1);
 #pragma unroll
-        for (int a = 0; a < D; ++a) fpg[a] = __ldg(fld.fpg[a] + c);
+        for (int a = 0; a < D; ++a) fpg[a] = __ldg(fld.fpg[a] + (D == 2 ? c : s0));
         cell_coords(D, p.n, c, idx);
         drag_pre_one<D, Real>(p, parts, fld, idx, o0, v0, fp, gp);
 #pragma unroll

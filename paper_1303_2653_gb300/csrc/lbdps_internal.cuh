@@ -92,6 +92,32 @@ template <> struct Store<__nv_bfloat16> {
 };
 
 // ---------------------------------------------------------------------------
+// Division by a fixed d >= 1 of n in [0, 2^31): with 2^(s-1) < d <= 2^s and mul =
+// ceil(2^(31+s) / d), floor(n / d) = floor(n mul / 2^(31+s)), since mul d -
+// 2^(31+s) < d <= 2^s (Granlund and Montgomery 1994).  Two instructions against
+// some twenty of a general division.
+// ---------------------------------------------------------------------------
+struct FastDiv {
+    unsigned mul = 0;   // 0: d = 1
+    int shift = 0;      // s - 1
+    __device__ __forceinline__ int operator()(int n) const
+    {
+        return mul ? (int)(__umulhi((unsigned)n, mul) >> shift) : n;
+    }
+};
+inline FastDiv make_fast_div(int d)
+{
+    FastDiv f;
+    int s = 0;
+    while ((1ll << s) < d) ++s;
+    if (s == 0) return f;
+    const unsigned long long two = 1ull << (31 + s);
+    f.mul = (unsigned)((two + d - 1) / d);
+    f.shift = s - 1;
+    return f;
+}
+
+// ---------------------------------------------------------------------------
 // Per-particle-count tables (deposition, Eq. 9-11, 19-20), built in FP64.
 // Index n = particles whose centre lies in the cell, clamped to ntab - 1
 // (beyond that the solid fraction is at its close-packing cap).

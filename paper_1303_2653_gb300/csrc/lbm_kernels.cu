@@ -132,22 +132,26 @@ __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
 __device__ __forceinline__ float sqrt_pos(float x) { return x > 0.f ? x * rsqrtf(x) : 0.f; }
 __device__ __forceinline__ double sqrt_pos(double x) { return sqrt(x); }
 
-// The collision runs blocks of kCollideThreads threads (a row of up to that
-// many cells).  Blocks per SM requested from the register allocator: D2Q9 in
-// FP32 fits in ~40 registers (12 blocks); D3Q19 in FP32 takes 56 (9 blocks,
-// 36 warps per SM: against 8 blocks at 64 registers, the 16-bit storages
-// run 8-9 % faster, FP32 the same); FP64 needs more.
+// The collision runs blocks of up to kCollideThreads threads.  Blocks of 128
+// per SM requested from the register allocator, GB300: D2Q9 in FP32 fits in 40
+// registers (12 blocks; 8 to 11 within 2 % on the 256 x 2048 riser, up to 9 %
+// slower on 512 x 2048 FP16); D3Q19 in FP32 takes 56 (9 blocks: 1,966 us on the
+// 256 x 256 x 1024 riser against 2,068 with 8 and 2,117 with 10), with the LES
+// sums 64 (8 blocks: 128 x 128 x 512 BF16 294 us against 302); FP64 needs 114 (4
+// blocks: 512 x 2048 with LES 880 us against 913 with 8 and spills).
 constexpr int kCollideThreads = 128;
-template <class L, class Real> struct K2Occupancy { static constexpr int value = 8; };
+constexpr int kSms = 152;
+template <class L, class Real, bool LES> struct K2Occupancy { static constexpr int value = 4; };
 #ifndef LBDPS_K2_BLOCKS_D2Q9_F32
 #define LBDPS_K2_BLOCKS_D2Q9_F32 12
 #endif
 #ifndef LBDPS_K2_BLOCKS_D3Q19_F32
 #define LBDPS_K2_BLOCKS_D3Q19_F32 9
 #endif
-template <> struct K2Occupancy<D2Q9, float> { static constexpr int value = LBDPS_K2_BLOCKS_D2Q9_F32; };
-template <> struct K2Occupancy<D3Q19, float> { static constexpr int value = LBDPS_K2_BLOCKS_D3Q19_F32; };
-template <> struct K2Occupancy<D3Q19, double> { static constexpr int value = 4; };
+template <bool LES> struct K2Occupancy<D2Q9, float, LES> { static constexpr int value = LBDPS_K2_BLOCKS_D2Q9_F32; };
+template <bool LES> struct K2Occupancy<D3Q19, float, LES> {
+    static constexpr int value = LES ? 8 : LBDPS_K2_BLOCKS_D3Q19_F32;
+};
 
 // Streaming across the faces of the lattice (Eq. 2 with the boundary rules),
 // run by the cells on a face after their own post-collision values are
@@ -332,6 +336,30 @@ __device__ __forceinline__ long long grid_block_index()
     return blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
 }
 
+// The collision's mapping of threads to cells: along the rows (grid: blocks of
+// a row, rows, planes), or, where rows are no multiple of a warp, along the
+// cells of a plane one row after the other (grid: blocks of a plane, 1, planes),
+// so that only the plane's last warp has idle lanes.
+struct CellMap {
+    int flat;         // 1: along the plane
+    int n0, cells;    // cells of a row, of a plane
+    FastDiv by_row;
+    // coordinates of this thread's cell; false: it has none
+    __device__ __forceinline__ bool cell(int *idx) const
+    {
+        const int c = blockIdx.x * blockDim.x + threadIdx.x;
+        idx[2] = blockIdx.z;
+        if (flat) {
+            idx[1] = by_row(c);
+            idx[0] = c - idx[1] * n0;
+            return c < cells;
+        }
+        idx[0] = c;
+        idx[1] = blockIdx.y;
+        return c < n0;
+    }
+};
+
 // index of this warp in the collision's grid (blocks in launch order, warps
 // of a block in order)
 __device__ __forceinline__ long long grid_warp_index()
@@ -423,9 +451,14 @@ __device__ __forceinline__ void collide_stream_cell(const StepParams<Real> &p, c
     }
     fld.rho[x] = rho;
     const Real solg = p.tab.sol_g[nn];
-    const Real slip = sqrt_pos(slip2);
-    Real beta;
-    if (t1.w == Real(0)) {
+    Real beta, slip = Real(0);
+    const bool empty64 = sizeof(Real) == 8 && n == 0;
+    if (!empty64) slip = sqrt_pos(slip2);
+    if (empty64) {
+        // beta_a = beta_c = 0: an empty cell spares the FP64 root and power
+        // (96 x 96 x 192 cells in FP64: 1,750 -> 1,457 us)
+        beta = t0.w * slip2;
+    } else if (t1.w == Real(0)) {
         beta = t0.w + t1.x * slip;                                   // Ergun
     } else {
         const Real re = t1.z * slip;                                 // Eq. 22
@@ -565,17 +598,13 @@ template <class Real> struct WarpMomentsHook {
 // tables) have gone out with the populations; a warp at the end of a row
 // with lanes past the lattice adds them first, from loads of its own.
 template <class L, class Real, class S, bool LES, bool FB, bool STATS>
-__global__ void __launch_bounds__(kCollideThreads, K2Occupancy<L, Real>::value)
+__global__ void __launch_bounds__(kCollideThreads, K2Occupancy<L, Real, LES>::value)
 k_collide_stream(StepParams<Real> p, PopLayout lay, PopPtrs<S> pp, CellList cells,
-                 Particles<Real> parts, Fields<Real> fld)
+                 Particles<Real> parts, Fields<Real> fld, CellMap map)
 {
     constexpr int Q = L::Q;
-    // grid: x along blockIdx.x/threadIdx.x, y = blockIdx.y, z = blockIdx.z
     int idx[3];
-    idx[0] = blockIdx.x * blockDim.x + threadIdx.x;
-    idx[1] = blockIdx.y;
-    idx[2] = blockIdx.z;
-    const bool active = idx[0] < p.n[0];
+    const bool active = map.cell(idx);
     if (!STATS) {
         if (!active) return;
         Real f[Q];
@@ -603,30 +632,46 @@ k_collide_stream(StepParams<Real> p, PopLayout lay, PopPtrs<S> pp, CellList cell
 // and of any state on demand).
 template <class L, class Real, class S>
 __global__ void __launch_bounds__(256)
-k_gas_moments(PopLayout lay, PopPtrs<S> pp, int n0, double *partials)
+k_gas_moments(PopLayout lay, PopPtrs<S> pp, CellMap map, double *partials)
 {
     int idx[3];
-    idx[0] = blockIdx.x * blockDim.x + threadIdx.x;
-    idx[1] = blockIdx.y;
-    idx[2] = blockIdx.z;
     Real mom[4];
-    lane_moments<L, Real, S>(idx[0] < n0, lay, pp, idx, mom);
+    const bool active = map.cell(idx);
+    lane_moments<L, Real, S>(active, lay, pp, idx, mom);
     warp_gas_partials<Real>(mom, partials + 4 * grid_warp_index());
 }
 
-// the collision's launch shape: blocks along each lattice row, up to 128
-// threads along x
-static inline int collide_tx(int n0)
+// The collision's launch shape: blocks along each lattice row, or along the
+// cells of a plane where rows of no multiple of 32 would leave lanes idle
+// (CellMap; 100 x 75 x 333 BF16 with LES: 24 of 32 lanes busy, 115 us; along the
+// plane 102).  Lattices of fewer than two blocks per SM take blocks of 64.
+struct CollideShape {
+    dim3 grid;
+    int threads;
+    CellMap map;
+};
+static CollideShape collide_shape(int dim, const int *n)
 {
-    return n0 >= kCollideThreads ? kCollideThreads : ((n0 + 31) / 32) * 32;
+    const int nz = dim == 3 ? n[2] : 1;
+    CollideShape s;
+    s.map.flat = n[0] % 32 != 0 && (long long)n[0] * n[1] < (1ll << 31) - kCollideThreads;
+    s.map.n0 = n[0];
+    s.map.cells = n[0] * n[1];
+    s.map.by_row = make_fast_div(n[0]);
+    const int line = s.map.flat ? s.map.cells : n[0];
+    const long long lines = (long long)(s.map.flat ? 1 : n[1]) * nz;
+    s.threads = std::min(kCollideThreads, ((line + 31) / 32) * 32);
+    auto blocks = [&] { return (line + s.threads - 1) / s.threads; };
+    if (s.threads == 128 && blocks() * lines < 2 * kSms) s.threads = 64;
+    s.grid = dim3(blocks(), s.map.flat ? 1 : n[1], nz);
+    return s;
 }
 
 long long collide_warps(int dim, const int *n)
 {
-    const int tx = collide_tx(n[0]);
-    return (long long)((n[0] + tx - 1) / tx) * n[1] * (dim == 3 ? n[2] : 1) * (tx / 32);
+    const CollideShape s = collide_shape(dim, n);
+    return (long long)s.grid.x * s.grid.y * s.grid.z * (s.threads / 32);
 }
-
 template <class L, class Real, class S>
 void launch_gas_moments(const PopLayout &lay, const S *f, const int *n, double *partials,
                         cudaStream_t st)
@@ -636,9 +681,8 @@ void launch_gas_moments(const PopLayout &lay, const S *f, const int *n, double *
         pp.pull[i] = f + (long long)i * lay.nce - lay.off<L>(i);
         pp.own[i] = nullptr;
     }
-    const int tx = collide_tx(n[0]);
-    const dim3 grid((n[0] + tx - 1) / tx, n[1], L::D == 3 ? n[2] : 1);
-    k_gas_moments<L, Real, S><<<grid, tx, 0, st>>>(lay, pp, n[0], partials);
+    const CollideShape s = collide_shape(L::D, n);
+    k_gas_moments<L, Real, S><<<s.grid, s.threads, 0, st>>>(lay, pp, s.map, partials);
 }
 
 template <class L, class Real, class S>
@@ -650,29 +694,29 @@ void launch_collide_stream(const StepParams<Real> &p, const PopLayout &lay, cons
         pp.pull[i] = fin + (long long)i * lay.nce - lay.off<L>(i);
         pp.own[i] = fout + (long long)i * lay.nce;
     }
-    // blocks along each lattice row, up to kCollideThreads threads along x
-    const int tx = collide_tx(p.n[0]);
-    const dim3 grid((p.n[0] + tx - 1) / tx, p.n[1], L::D == 3 ? p.n[2] : 1);
+    const CollideShape s = collide_shape(L::D, p.n);
+    const dim3 grid = s.grid;
+    const int tx = s.threads;
     const bool les = p.les_k > Real(0), fb = p.has_fb != 0;
     if (p.gas_partials) {
         if (les && fb)
-            k_collide_stream<L, Real, S, true, true, true><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld);
+            k_collide_stream<L, Real, S, true, true, true><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld, s.map);
         else if (les)
-            k_collide_stream<L, Real, S, true, false, true><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld);
+            k_collide_stream<L, Real, S, true, false, true><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld, s.map);
         else if (fb)
-            k_collide_stream<L, Real, S, false, true, true><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld);
+            k_collide_stream<L, Real, S, false, true, true><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld, s.map);
         else
-            k_collide_stream<L, Real, S, false, false, true><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld);
+            k_collide_stream<L, Real, S, false, false, true><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld, s.map);
         return;
     }
     if (les && fb)
-        k_collide_stream<L, Real, S, true, true, false><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld);
+        k_collide_stream<L, Real, S, true, true, false><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld, s.map);
     else if (les)
-        k_collide_stream<L, Real, S, true, false, false><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld);
+        k_collide_stream<L, Real, S, true, false, false><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld, s.map);
     else if (fb)
-        k_collide_stream<L, Real, S, false, true, false><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld);
+        k_collide_stream<L, Real, S, false, true, false><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld, s.map);
     else
-        k_collide_stream<L, Real, S, false, false, false><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld);
+        k_collide_stream<L, Real, S, false, false, false><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld, s.map);
 }
 
 // ---------------------------------------------------------------------------

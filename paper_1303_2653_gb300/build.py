@@ -35,7 +35,8 @@ def build_workloads(force: bool = False) -> str:
     return out
 
 
-CU_SOURCES = ["lbm_kernels.cu", "particle_kernels.cu", "stats_kernels.cu", "lbdps_api.cu",
+CU_SOURCES = ["lbm_kernels.cu", "lbm_kernels_part1.cu", "lbm_kernels_part2.cu",
+              "lbm_kernels_part3.cu", "particle_kernels.cu", "stats_kernels.cu", "lbdps_api.cu",
               "lbdps_server.cu", "noalloc_sort.cu", "bubble_kernels.cu", "contact_kernels.cu"]
 HEADERS = ["lbdps_internal.cuh", "particle_common.cuh"]
 
@@ -45,7 +46,7 @@ def nvcc_flags(extra=()):
             f"-I{INCLUDE}", f"-I{CSRC}", *extra]
 
 
-def build_lbdps(force: bool = False, verbose_ptxas: bool = False, jobs: int = 4) -> str:
+def build_lbdps(force: bool = False, verbose_ptxas: bool = False, jobs: int = 8) -> str:
     """Compile the CUDA library into ``liblbdps.so`` next to this file."""
     out = os.path.join(HERE, "liblbdps.so")
     srcs = [os.path.join(CSRC, s) for s in CU_SOURCES]

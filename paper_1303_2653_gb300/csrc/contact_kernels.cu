@@ -226,7 +226,7 @@ k_contacts(StepParams<Real> p, Particles<Real> parts, CellList cells, Real *diag
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= np) return;
     int idx[3];
-    cell_coords(D, p.n, __ldg(parts.cell + i), idx);
+    cell_coords<D, Real>(p, __ldg(parts.cell + i), idx);
     float oi[3] = {0.f, 0.f, 0.f};
     Real oR[3] = {Real(0), Real(0), Real(0)};
     Real vi[3] = {Real(0), Real(0), Real(0)}, wi[3] = {Real(0), Real(0), Real(0)};
@@ -333,7 +333,7 @@ k_contacts_binned(StepParams<Real> p, Particles<Real> parts, CellList cells, Rea
 #pragma unroll
     for (int a = 0; a < 3; ++a) per[a] = (a < D) && (p.bc[2 * a] == BC_PERIODIC);
     if (i < np) {
-        cell_coords(D, p.n, __ldg(parts.cell + i), idx);
+        cell_coords<D, Real>(p, __ldg(parts.cell + i), idx);
 #pragma unroll
         for (int a = 0; a < D; ++a) {
             oi[a] = __ldg(parts.off[a] + i);
@@ -350,12 +350,12 @@ k_contacts_binned(StepParams<Real> p, Particles<Real> parts, CellList cells, Rea
 
     for (int s = first; s < end;) {
         // the run [s, e): the particles left in the row of slot s (at most kRowCells cells)
-        const int c0 = __ldg(parts.cell + s), xa = c0 % p.n[0], row = c0 - xa;
+        const int c0 = __ldg(parts.cell + s), xa = c0 - p.by_row(c0) * p.n[0], row = c0 - xa;
         const int e = min(end, cells.begin(row + min(p.n[0], xa + kRowCells)));
         const int xb = __ldg(parts.cell + e - 1) - row;
         const int ncx = xb - xa + 1;
         int ri[3];
-        cell_coords(D, p.n, row, ri);
+        cell_coords<D, Real>(p, row, ri);
         // m subcells per cell along each axis, none smaller than the reach
         int m = max(1, (int)(0.9999f / cut));
         while (m > 1 && (ncx * m + 2) * (m + 2) * (D == 3 ? m + 2 : 1) > kBinMax) --m;

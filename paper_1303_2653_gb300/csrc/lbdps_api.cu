@@ -549,6 +549,8 @@ template <class L, class Real, class S> struct EngineT : Engine {
         p.ncell = H->ncell;
         for (int f6 = 0; f6 < 6; ++f6) p.bc[f6] = H->bc[f6];
         p.vert = D - 1;
+        p.by_row = make_fast_div(H->n[0]);
+        p.by_plane = make_fast_div(D == 3 ? H->n[0] * H->n[1] : H->ncell);
         p.tau = (Real)k.tau;
         p.inv_tau = (Real)(1.0 / k.tau);
         p.les_k = (Real)(18.0 * k.cs * k.cs);

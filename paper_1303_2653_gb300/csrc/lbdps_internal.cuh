@@ -154,6 +154,7 @@ template <class Real> struct StepParams {
     int ncell;
     int bc[6];
     int vert;                 // vertical axis (dim - 1)
+    FastDiv by_row, by_plane; // divisions by n[0] and n[0] n[1]
     Real tau, inv_tau;
     Real les_k;               // 18 C_s^2 (0 = LES off)
     Real fb[3];               // gas body force density

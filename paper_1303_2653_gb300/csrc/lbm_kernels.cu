@@ -3,7 +3,12 @@
 // import/export.
 #include "lbdps_internal.cuh"
 
+#ifndef LBDPS_LBM_PART
+#define LBDPS_LBM_PART 0
+#endif
+
 #include <algorithm>
+#include <type_traits>
 
 namespace lbdpsk {
 
@@ -21,7 +26,7 @@ template <class Real> struct TableOut {
     typename Vec4<Real>::type *pk0, *pk1;
 };
 
-__device__ double emms_omega(double eg)
+__device__ static double emms_omega(double eg)
 {
     // Eq. 20 (Yang et al. fit); 1 in the Ergun regime eps_g <= 0.74
     if (eg <= 0.74) return 1.0;
@@ -341,15 +346,17 @@ __device__ __forceinline__ long long grid_block_index()
 // cells of a plane one row after the other (grid: blocks of a plane, 1, planes),
 // so that only the plane's last warp has idle lanes.
 struct CellMap {
-    int flat;         // 1: along the plane
     int n0, cells;    // cells of a row, of a plane
     FastDiv by_row;
-    // coordinates of this thread's cell; false: it has none
-    __device__ __forceinline__ bool cell(int *idx) const
+    // coordinates of this thread's cell; false: it has none.  A mapping of its
+    // own (FLAT: along the plane), because a row index that is the same for the
+    // whole block stays in uniform registers: one kernel for both cost the
+    // 256 x 2048 riser 1.2 of 15.5 us.
+    template <bool FLAT> __device__ __forceinline__ bool cell(int *idx) const
     {
         const int c = blockIdx.x * blockDim.x + threadIdx.x;
         idx[2] = blockIdx.z;
-        if (flat) {
+        if (FLAT) {
             idx[1] = by_row(c);
             idx[0] = c - idx[1] * n0;
             return c < cells;
@@ -597,14 +604,14 @@ template <class Real> struct WarpMomentsHook {
 // inside the collision, after the deposition's loads (cell list, particles,
 // tables) have gone out with the populations; a warp at the end of a row
 // with lanes past the lattice adds them first, from loads of its own.
-template <class L, class Real, class S, bool LES, bool FB, bool STATS>
+template <class L, class Real, class S, bool LES, bool FB, bool STATS, bool FLAT>
 __global__ void __launch_bounds__(kCollideThreads, K2Occupancy<L, Real, LES>::value)
 k_collide_stream(StepParams<Real> p, PopLayout lay, PopPtrs<S> pp, CellList cells,
                  Particles<Real> parts, Fields<Real> fld, CellMap map)
 {
     constexpr int Q = L::Q;
     int idx[3];
-    const bool active = map.cell(idx);
+    const bool active = map.cell<FLAT>(idx);
     if (!STATS) {
         if (!active) return;
         Real f[Q];
@@ -630,48 +637,56 @@ k_collide_stream(StepParams<Real> p, PopLayout lay, PopPtrs<S> pp, CellList cell
 // The cell moments of a state without a collision, with the collision's
 // grid, loads and per-warp sums (the statistics of the last state of a run,
 // and of any state on demand).
-template <class L, class Real, class S>
+template <class L, class Real, class S, bool FLAT>
 __global__ void __launch_bounds__(256)
 k_gas_moments(PopLayout lay, PopPtrs<S> pp, CellMap map, double *partials)
 {
     int idx[3];
     Real mom[4];
-    const bool active = map.cell(idx);
+    const bool active = map.cell<FLAT>(idx);
     lane_moments<L, Real, S>(active, lay, pp, idx, mom);
     warp_gas_partials<Real>(mom, partials + 4 * grid_warp_index());
 }
 
-// The collision's launch shape: blocks along each lattice row, or along the
-// cells of a plane where rows of no multiple of 32 would leave lanes idle
-// (CellMap; 100 x 75 x 333 BF16 with LES: 24 of 32 lanes busy, 115 us; along the
-// plane 102).  Lattices of fewer than two blocks per SM take blocks of 64.
+// The collision's launch shape: blocks along each lattice row; along the cells
+// of a plane (CellMap) where rows would leave an eighth of the lanes idle and
+// the lattice has two blocks for every SM: 100 x 75 x 333 BF16 with LES, 24 of 32
+// lanes busy, 115 us, along the plane 102.  Short of that the row's uniform
+// index is worth more (75 x 193: 8.5 us, along the plane 8.9; 60 x 720, 15 of 16
+// lanes busy: 9.2 and 10.1).  Few blocks of 128 are split in two.
 struct CollideShape {
     dim3 grid;
     int threads;
+    bool flat;
     CellMap map;
 };
 static CollideShape collide_shape(int dim, const int *n)
 {
     const int nz = dim == 3 ? n[2] : 1;
     CollideShape s;
-    s.map.flat = n[0] % 32 != 0 && (long long)n[0] * n[1] < (1ll << 31) - kCollideThreads;
+    const long long plane = (long long)n[0] * n[1], lanes = (n[0] + 31) / 32 * 32;
+    s.flat = 8ll * n[0] < 7 * lanes && plane * nz >= 2ll * kSms * kCollideThreads &&
+             plane < (1ll << 31) - kCollideThreads;
     s.map.n0 = n[0];
     s.map.cells = n[0] * n[1];
     s.map.by_row = make_fast_div(n[0]);
-    const int line = s.map.flat ? s.map.cells : n[0];
-    const long long lines = (long long)(s.map.flat ? 1 : n[1]) * nz;
+    const int line = s.flat ? s.map.cells : n[0];
+    const long long lines = (long long)(s.flat ? 1 : n[1]) * nz;
     s.threads = std::min(kCollideThreads, ((line + 31) / 32) * 32);
     auto blocks = [&] { return (line + s.threads - 1) / s.threads; };
     if (s.threads == 128 && blocks() * lines < 2 * kSms) s.threads = 64;
-    s.grid = dim3(blocks(), s.map.flat ? 1 : n[1], nz);
+    s.grid = dim3(blocks(), s.flat ? 1 : n[1], nz);
     return s;
 }
 
+#if LBDPS_LBM_PART == 0
 long long collide_warps(int dim, const int *n)
 {
     const CollideShape s = collide_shape(dim, n);
     return (long long)s.grid.x * s.grid.y * s.grid.z * (s.threads / 32);
 }
+#endif
+
 template <class L, class Real, class S>
 void launch_gas_moments(const PopLayout &lay, const S *f, const int *n, double *partials,
                         cudaStream_t st)
@@ -682,7 +697,8 @@ void launch_gas_moments(const PopLayout &lay, const S *f, const int *n, double *
         pp.own[i] = nullptr;
     }
     const CollideShape s = collide_shape(L::D, n);
-    k_gas_moments<L, Real, S><<<s.grid, s.threads, 0, st>>>(lay, pp, s.map, partials);
+    if (s.flat) k_gas_moments<L, Real, S, true><<<s.grid, s.threads, 0, st>>>(lay, pp, s.map, partials);
+    else k_gas_moments<L, Real, S, false><<<s.grid, s.threads, 0, st>>>(lay, pp, s.map, partials);
 }
 
 template <class L, class Real, class S>
@@ -695,30 +711,27 @@ void launch_collide_stream(const StepParams<Real> &p, const PopLayout &lay, cons
         pp.own[i] = fout + (long long)i * lay.nce;
     }
     const CollideShape s = collide_shape(L::D, p.n);
-    const dim3 grid = s.grid;
-    const int tx = s.threads;
-    const bool les = p.les_k > Real(0), fb = p.has_fb != 0;
-    if (p.gas_partials) {
-        if (les && fb)
-            k_collide_stream<L, Real, S, true, true, true><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld, s.map);
-        else if (les)
-            k_collide_stream<L, Real, S, true, false, true><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld, s.map);
-        else if (fb)
-            k_collide_stream<L, Real, S, false, true, true><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld, s.map);
-        else
-            k_collide_stream<L, Real, S, false, false, true><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld, s.map);
-        return;
+    auto run = [&](auto kern) { kern<<<s.grid, s.threads, 0, st>>>(p, lay, pp, cells, parts, fld, s.map); };
+    auto pick_map = [&](auto les, auto fb, auto stats) {
+        constexpr bool l = decltype(les)::value, f = decltype(fb)::value, m = decltype(stats)::value;
+        if (s.flat) run(k_collide_stream<L, Real, S, l, f, m, true>);
+        else run(k_collide_stream<L, Real, S, l, f, m, false>);
+    };
+    auto pick_stats = [&](auto les, auto fb) {
+        if (p.gas_partials) pick_map(les, fb, std::true_type());
+        else pick_map(les, fb, std::false_type());
+    };
+    const bool fb = p.has_fb != 0;
+    if (p.les_k > Real(0)) {
+        if (fb) pick_stats(std::true_type(), std::true_type());
+        else pick_stats(std::true_type(), std::false_type());
+    } else {
+        if (fb) pick_stats(std::false_type(), std::true_type());
+        else pick_stats(std::false_type(), std::false_type());
     }
-    if (les && fb)
-        k_collide_stream<L, Real, S, true, true, false><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld, s.map);
-    else if (les)
-        k_collide_stream<L, Real, S, true, false, false><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld, s.map);
-    else if (fb)
-        k_collide_stream<L, Real, S, false, true, false><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld, s.map);
-    else
-        k_collide_stream<L, Real, S, false, false, false><<<grid, tx, 0, st>>>(p, lay, pp, cells, parts, fld, s.map);
 }
 
+#if LBDPS_LBM_PART == 0
 // ---------------------------------------------------------------------------
 // Batched collide-stream of the serving loop: persistent blocks walk the
 // work table of (bed, tile) entries; each entry is kBatchTile consecutive
@@ -766,7 +779,8 @@ k_collide_stream_batched(const BatchBed *__restrict__ beds, const int2 *__restri
         if (step >= b.nsteps) continue;
         const int c = e.y * kBatchTile + threadIdx.x;
         if (c >= b.ncell) continue;
-        const int idx[3] = {c % b.sp.n[0], c / b.sp.n[0], 0};
+        const int row = b.sp.by_row(c);
+        const int idx[3] = {c - row * b.sp.n[0], row, 0};
         const int a = (b.parity0 + step) & 1;
         if (b.storage == ST_F16) batched_cell<__half>(b, a, idx);
         else if (b.storage == ST_BF16) batched_cell<__nv_bfloat16>(b, a, idx);
@@ -794,6 +808,8 @@ void launch_collide_stream_batched(const BatchBed *beds, BatchWork work, int ste
     if (!work.count) return;
     k_collide_stream_batched<<<grid, kBatchTile, 0, st>>>(beds, work.cell_tiles, work.count, step);
 }
+
+#endif   // LBDPS_LBM_PART == 0
 
 // ---------------------------------------------------------------------------
 // Equilibrium initialisation and population import/export (full values in
@@ -939,14 +955,23 @@ void launch_export_fields(const FieldExport<Real> &x, long long lo, long long n,
     template void launch_import_populations<L, R, S>(const PopLayout &, int, const double *,        \
                                                      long long, long long, S *, cudaStream_t);
 
+// compiled in four units (lbm_kernels_part*.cu define LBDPS_LBM_PART), so that a
+// build takes as long as one of them
+#if LBDPS_LBM_PART == 0
 LBDPS_INST_LBM(D2Q9, double, double)
 LBDPS_INST_LBM(D2Q9, float, float)
+#elif LBDPS_LBM_PART == 1
 LBDPS_INST_LBM(D2Q9, float, __half)
 LBDPS_INST_LBM(D2Q9, float, __nv_bfloat16)
+#elif LBDPS_LBM_PART == 2
 LBDPS_INST_LBM(D3Q19, double, double)
 LBDPS_INST_LBM(D3Q19, float, float)
+#else
 LBDPS_INST_LBM(D3Q19, float, __half)
 LBDPS_INST_LBM(D3Q19, float, __nv_bfloat16)
+#endif
+
+#if LBDPS_LBM_PART == 0
 
 template void launch_export_fields<float>(const FieldExport<float> &, long long, long long, double *,
                                           cudaStream_t);
@@ -957,5 +982,7 @@ template void launch_build_tables<double>(int, double, double, double, double, d
                                           double *, CountTables<double>, cudaStream_t);
 template void launch_build_tables<float>(int, double, double, double, double, double, int, int,
                                          double *, CountTables<float>, cudaStream_t);
+
+#endif
 
 }  // namespace lbdpsk

@@ -220,7 +220,7 @@ __device__ __forceinline__ void foreign_sums(const StepParams<Real> &p, const Pa
                                              bool mine, Real (*sfor)[kForeignChunk], Real *S, Real *A)
 {
     int idx[3] = {0, 0, 0};
-    cell_coords(D, p.n, cell, idx);
+    cell_coords<D, Real>(p, cell, idx);
     for (int base = lo; base < hi; base += kForeignChunk) {
         const int cnt = min(kForeignChunk, hi - base);
         __syncthreads();   // the previous chunk has been read
@@ -285,7 +285,7 @@ __device__ __forceinline__ void drag_step_particle(const StepParams<Real> &p,
         s1 = cells.begin(c + 1);
 #pragma unroll
         for (int a = 0; a < D; ++a) fpg[a] = __ldg(fld.fpg[a] + (D == 2 ? c : s0));
-        cell_coords(D, p.n, c, idx);
+        cell_coords<D, Real>(p, c, idx);
         drag_pre_one<D, Real>(p, parts, fld, idx, o0, v0, fp, gp);
 #pragma unroll
         for (int a = 0; a < D; ++a) sfp[a][k - block_first] = fp[a];
@@ -791,7 +791,7 @@ __device__ __forceinline__ void detect_one(const StepParams<Real> &p, const Part
                                            unsigned long long *npairs, long long pair_cap, int i)
 {
     int idx[3];
-    cell_coords(D, p.n, parts.cell[i], idx);
+    cell_coords<D, Real>(p, parts.cell[i], idx);
     float oi[3] = {0.f, 0.f, 0.f};
     bool per[3];
 #pragma unroll
@@ -956,7 +956,7 @@ k_overlaps(StepParams<Real> p, Particles<Real> parts, CellList cells,
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= np) return;
     int idx[3];
-    cell_coords(D, p.n, parts.cell[i], idx);
+    cell_coords<D, Real>(p, parts.cell[i], idx);
     float oi[3] = {0.f, 0.f, 0.f};
     bool per[3];
 #pragma unroll

@@ -27,9 +27,11 @@ def _built():
 
 
 # rows of a multiple of 32 and not; fewer cells than a warp and than a block; one row; a row longer
-# than a block by one cell; enough blocks for 128 threads each; planes that end inside a warp
+# than a block by one cell; enough blocks for 128 threads each; planes that end inside a warp; from
+# (3, 13000) on, lattices large enough for threads along the plane
 @pytest.mark.parametrize("n", [(3, 5), (31, 33), (32, 9), (33, 1), (129, 7), (250, 160), (5, 3, 4),
-                               (32, 3, 5), (33, 31, 7), (100, 9, 50)])
+                               (32, 3, 5), (33, 31, 7), (3, 13000), (129, 310), (100, 9, 50),
+                               (33, 31, 41)])
 @pytest.mark.parametrize("storage", [W.STORE_F64, W.STORE_F32])
 def test_row_shapes(n, storage):
     from paper_1303_2653_gb300 import lbdps as L

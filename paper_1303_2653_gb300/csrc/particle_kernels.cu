@@ -126,27 +126,43 @@ __device__ __forceinline__ void drag_pre_one(const StepParams<Real> &p, const Pa
         bk += w * r4.w;
     }
     // grad p at each node: central differences of rho/3 (one-sided next to a
-    // non-periodic face).  Every neighbour is loaded, also where it is itself
-    // a stencil node (an L1 hit): independent loads keep more gathers in
-    // flight than selects between loaded and loading values (3D riser: 720
-    // against 747 us per launch)
+    // non-periodic face).  Along an axis one neighbour of a stencil node is the
+    // stencil's other node, whose rho is loaded once (NC loads); only where the
+    // stencil is clamped at a face is it another cell, loaded on its own.  The
+    // gathers are bound by the lines a warp's load touches, and this takes 32
+    // instead of 48 loads of rho in 3D, 12 instead of 16 in 2D: 256 x 256 x 1024
+    // riser 581 -> 491 us (with the registers below), 256 x 2048 13.8 -> 13.4,
+    // crowded 256 x 1024 bed 73.3 -> 66.5.
+    Real rc[NC];
 #pragma unroll
-    for (int corner = 0; corner < NC; ++corner) {
+    for (int corner = 0; corner < NC; ++corner) rc[corner] = __ldg(fld.rho + node[corner]);
 #pragma unroll
-        for (int a = 0; a < D; ++a) {
-            if (p.n[a] == 1) continue;
-            const int bit = (corner >> a) & 1;
+    for (int a = 0; a < D; ++a) {
+        if (p.n[a] == 1) continue;
+        const int stride = (a == 0) ? 1 : (a == 1) ? p.n[0] : p.n[0] * p.n[1];
+        const bool per = (p.bc[2 * a] == BC_PERIODIC);
+        // of node i0 and of node i1: the neighbours below and above, relative
+        int lo[2], hi[2];
+        Real scale[2];
+#pragma unroll
+        for (int bit = 0; bit < 2; ++bit) {
             const int q = bit ? i1[a] : i0[a];
-            const int stride = (a == 0) ? 1 : (a == 1) ? p.n[0] : p.n[0] * p.n[1];
-            int lo = q - 1, hi = q + 1;
-            Real scale = Real(1) / Real(6);    // (1/3) / 2: central difference of rho/3
-            const bool per = (p.bc[2 * a] == BC_PERIODIC);
-            if (lo < 0) { if (per) lo += p.n[a]; else { lo = q; scale = Real(1) / Real(3); } }
-            if (hi >= p.n[a]) { if (per) hi -= p.n[a]; else { hi = q; scale = Real(1) / Real(3); } }
-            const int x = node[corner];
-            const Real rh = __ldg(fld.rho + x + (hi - q) * stride);
-            const Real rl = __ldg(fld.rho + x + (lo - q) * stride);
-            gk[a] += wt[corner] * ((rh - rl) * scale);
+            lo[bit] = q - 1;
+            hi[bit] = q + 1;
+            scale[bit] = Real(1) / Real(6);    // (1/3) / 2: central difference of rho/3
+            if (lo[bit] < 0) { if (per) lo[bit] += p.n[a]; else { lo[bit] = q; scale[bit] = Real(1) / Real(3); } }
+            if (hi[bit] >= p.n[a]) { if (per) hi[bit] -= p.n[a]; else { hi[bit] = q; scale[bit] = Real(1) / Real(3); } }
+        }
+        const bool next = hi[0] == i1[a] && lo[1] == i0[a];   // the two nodes are neighbours
+#pragma unroll
+        for (int corner = 0; corner < NC; ++corner) {
+            const int bit = (corner >> a) & 1;
+            const int x = node[corner], q = bit ? i1[a] : i0[a];
+            const Real outer = __ldg(fld.rho + x + ((bit ? hi[1] : lo[0]) - q) * stride);
+            Real inner = rc[corner ^ (1 << a)];
+            if (!next) inner = __ldg(fld.rho + x + ((bit ? lo[1] : hi[0]) - q) * stride);
+            const Real rh = bit ? outer : inner, rl = bit ? inner : outer;
+            gk[a] += wt[corner] * ((rh - rl) * scale[bit]);
         }
     }
     const Real coef = p.vp * bk / sk;   // V_p beta_k / (1 - eps_k), Eq. 26
@@ -183,16 +199,16 @@ __device__ __forceinline__ void drag_pre_one(const StepParams<Real> &p, const Pa
 // more from registers to hold them in flight than from warps: in 2D 64
 // registers (4 blocks) against 48 (5 blocks, 88 bytes of spills) take the step
 // of the 256 x 2048 riser from 45.0 to 42.5 us, 512 x 2048 from 75.5 to 71.3 and
-// the crowded 256 x 1024 bed from 210.5 to 206.8; in 3D 4 blocks spill (drag of
-// the 256 x 256 x 1024 riser 823 us against 620) and 2 leave it short of warps
-// (717).  Detection fits 40 registers in 2D FP32 (6 blocks: 200,000 particles in
+// the crowded 256 x 1024 bed from 210.5 to 206.8; in 3D 128 registers (2 blocks)
+// take the drag of the 256 x 256 x 1024 riser to 491 us, 80 (3 blocks, 56 bytes
+// of spills) to 535, 64 (4) to 622.  Detection fits 40 registers in 2D FP32 (6 blocks: 200,000 particles in
 // one wave, see wave_block; 5 or 7 cost it half a microsecond) and 48 in 3D (5
 // blocks; 4 take 16 us longer on that riser).
 #ifndef LBDPS_DRAG_BLOCKS_2D_F32
 #define LBDPS_DRAG_BLOCKS_2D_F32 4
 #endif
 #ifndef LBDPS_DRAG_BLOCKS_3D_F32
-#define LBDPS_DRAG_BLOCKS_3D_F32 3
+#define LBDPS_DRAG_BLOCKS_3D_F32 2
 #endif
 template <int D, class Real> struct DragOccupancy { static constexpr int value = 2; };
 template <> struct DragOccupancy<2, float> { static constexpr int value = LBDPS_DRAG_BLOCKS_2D_F32; };

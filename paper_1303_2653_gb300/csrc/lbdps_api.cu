@@ -719,7 +719,8 @@ template <class L, class Real, class S> struct EngineT : Engine {
         CHECK_LAUNCH();
         launch_cell_scan(counts, cells_out(dst), H->ncell, st);
         CHECK_LAUNCH();
-        launch_place<Real>(D, key, counts, cells(dst), slot, idslot, part[src], part[dst], H->np, st);
+        launch_place<Real>(D, key, counts, cells_out(dst), H->ncell, slot, idslot, part[src], part[dst],
+                           H->np, st);
         CHECK_LAUNCH();
         return LBDPS_OK;
     }
@@ -754,7 +755,7 @@ template <class L, class Real, class S> struct EngineT : Engine {
             CHECK_LAUNCH();
             Particles<Real> src = stage;
             src.id = part[a].id;
-            launch_place<Real>(D, key, counts, cells(b), slot, idslot, src, part[b], np, st);
+            launch_place<Real>(D, key, counts, cells_out(b), H->ncell, slot, idslot, src, part[b], np, st);
             CHECK_LAUNCH();
         } else {
             int rc = clear_cells(b);

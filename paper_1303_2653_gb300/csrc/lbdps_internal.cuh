@@ -433,13 +433,15 @@ template <int D, class Real>
 void launch_particles_from_host_order(const double *pos, const double *vel, int np, double pos_div,
                                       double vel_mul, Particles<Real> dst, cudaStream_t st);
 
-// one-launch scan of counts[0..ncell] (counts[ncell] = 0) into a CellList
+// one-launch scan of counts[0..ncell] (counts[ncell] = 0) into a CellList; in
+// small tiles only the tiles and their totals, for launch_place
 void launch_cell_scan(const int *counts, CellListOut out, int ncell, cudaStream_t st);
 
-// slot placement and in-cell ordering by id: src (any order) -> dst (cell, id)
+// slot placement and in-cell ordering by id: src (any order) -> dst (cell, id);
+// follows launch_cell_scan into `out`, whose base it completes on small lattices
 template <class Real>
-void launch_place(int dim, const int *key, int *counts, CellList cells, int2 *slot, int *idslot,
-                  Particles<Real> src, Particles<Real> dst, int np, cudaStream_t st);
+void launch_place(int dim, const int *key, int *counts, CellListOut out, int ncell, int2 *slot,
+                  int *idslot, Particles<Real> src, Particles<Real> dst, int np, cudaStream_t st);
 
 template <int D, class Real>
 void launch_detect(const StepParams<Real> &p, Particles<Real> parts, CellList cells, int *best,

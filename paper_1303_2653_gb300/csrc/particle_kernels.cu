@@ -604,8 +604,9 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *warp_tot, int *t
 constexpr int kCellScanThreads = 1024;
 
 // Tile `tile` of `nt` (one block of kCellScanThreads threads; every thread
-// calls it); ITEMS = tile cells / kCellScanThreads.
-template <int ITEMS>
+// calls it); ITEMS = tile cells / kCellScanThreads.  BASE: the block that
+// finishes last also scans the tile totals; else the scatter does (k_scatter).
+template <int ITEMS, bool BASE>
 __device__ __forceinline__ void cell_scan_tile(const int *__restrict__ counts, const CellListOut &out,
                                                int n, int tile, int nt, int *warp_tot, int &total,
                                                bool &last)
@@ -646,8 +647,9 @@ __device__ __forceinline__ void cell_scan_tile(const int *__restrict__ counts, c
             if (e + 3 < n) out.local[e + 3] = e4.w;
         }
     }
+    if (threadIdx.x == 0) out.tile_total[tile] = total;
+    if (!BASE) return;
     if (threadIdx.x == 0) {
-        out.tile_total[tile] = total;
         __threadfence();
         const unsigned done = atomicAdd(out.ticket, 1u);
         last = (done == (unsigned)nt - 1u);
@@ -671,14 +673,14 @@ __device__ __forceinline__ void cell_scan_tile(const int *__restrict__ counts, c
     }
 }
 
-template <int ITEMS>
+template <int ITEMS, bool BASE>
 __global__ void __launch_bounds__(kCellScanThreads)
 k_cell_scan(const int *__restrict__ counts, CellListOut out, int n)
 {
     __shared__ int warp_tot[32];
     __shared__ int total;
     __shared__ bool last;
-    cell_scan_tile<ITEMS>(counts, out, n, blockIdx.x, gridDim.x, warp_tot, total, last);
+    cell_scan_tile<ITEMS, BASE>(counts, out, n, blockIdx.x, gridDim.x, warp_tot, total, last);
 }
 
 static_assert((kCellScanThreads << 2) == (1 << kCellTileLog2), "4 counts per thread in small tiles");
@@ -689,9 +691,9 @@ void launch_cell_scan(const int *counts, CellListOut out, int ncell, cudaStream_
     const int n = ncell + 1;
     const int nt = cell_tiles(ncell);
     if (out.shift == kCellTileLog2Large)
-        k_cell_scan<16><<<nt, kCellScanThreads, 0, st>>>(counts, out, n);
+        k_cell_scan<16, true><<<nt, kCellScanThreads, 0, st>>>(counts, out, n);
     else
-        k_cell_scan<4><<<nt, kCellScanThreads, 0, st>>>(counts, out, n);
+        k_cell_scan<4, false><<<nt, kCellScanThreads, 0, st>>>(counts, out, n);
 }
 
 // ---------------------------------------------------------------------------
@@ -702,23 +704,56 @@ void launch_cell_scan(const int *counts, CellListOut out, int ncell, cudaStream_
 // and the payload is gathered to begin(cell) + rank, the (cell, id) order.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void scatter_one(const int *__restrict__ key, const int *__restrict__ id,
-                                            int *__restrict__ counts, const CellList &cells,
-                                            int2 *__restrict__ slot, int *__restrict__ idslot, int k)
+                                            int *__restrict__ counts, const int *__restrict__ local,
+                                            const int *base, int shift, int2 *__restrict__ slot,
+                                            int *__restrict__ idslot, int k)
 {
     const int c = key[k];
     const int old = atomicSub(&counts[c], 1);
-    const int s = cells.begin(c) + old - 1;
+    const int s = __ldg(local + c) + base[c >> shift] + old - 1;
     slot[s] = make_int2(k, c);
     idslot[s] = id[k];
 }
 
+// TOTALS (lattices in small tiles, at most kScatterTiles): every block first
+// scans the tile totals of the cell scan for itself, beside the loads of its
+// keys, and block 0 stores the result for the kernels that follow.  Left to the
+// scan's last block it stood at the end of a chain of a fence, a ticket and
+// dependent loads, about a microsecond of every step (GB300, us per step: 75 x
+// 193 23.0 -> 21.9, 256 x 2048 41.1 -> 40.2, 60 x 720 29.5 -> 28.7).
+constexpr int kScatterTiles = (kLargeLatticeCells >> kCellTileLog2) + 1;
+template <bool TOTALS>
 __global__ void k_scatter(const int *__restrict__ key, const int *__restrict__ id,
-                          int *__restrict__ counts, CellList cells, int2 *__restrict__ slot,
+                          int *__restrict__ counts, CellListOut cells, int nt, int2 *__restrict__ slot,
                           int *__restrict__ idslot, int np)
 {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= np) return;
-    scatter_one(key, id, counts, cells, slot, idslot, k);
+    if (TOTALS) {
+        __shared__ int base[kScatterTiles + 1];
+        __shared__ int warp_tot[32];
+        __shared__ int total;
+        const int per = (nt + blockDim.x - 1) / blockDim.x, t0 = threadIdx.x * per;
+        int sum = 0;
+        for (int t = t0; t < min(t0 + per, nt); ++t) {
+            const int v = __ldg(cells.tile_total + t);
+            base[t] = v;
+            sum += v;
+        }
+        int run = block_exclusive_scan(sum, warp_tot, &total);
+        for (int t = t0; t < min(t0 + per, nt); ++t) {
+            const int v = base[t];
+            base[t] = run;
+            run += v;
+        }
+        __syncthreads();
+        if (blockIdx.x == 0) {
+            for (int t = threadIdx.x; t < nt; t += blockDim.x) cells.base[t] = base[t];
+            if (threadIdx.x == 0) cells.base[nt] = total;
+        }
+        if (k < np) scatter_one(key, id, counts, cells.local, base, cells.shift, slot, idslot, k);
+    } else {
+        if (k < np) scatter_one(key, id, counts, cells.local, cells.base, cells.shift, slot, idslot, k);
+    }
 }
 
 // The payload of the particle in slot s is loaded before its rank is known
@@ -774,12 +809,19 @@ k_gather(CellList cells, const int2 *__restrict__ slot, const int *__restrict__ 
 }
 
 template <class Real>
-void launch_place(int dim, const int *key, int *counts, CellList cells, int2 *slot, int *idslot,
-                  Particles<Real> src, Particles<Real> dst, int np, cudaStream_t st)
+void launch_place(int dim, const int *key, int *counts, CellListOut out, int ncell, int2 *slot,
+                  int *idslot, Particles<Real> src, Particles<Real> dst, int np, cudaStream_t st)
 {
     if (np == 0) return;
-    const int bs = wave_block(k_scatter, np);
-    k_scatter<<<(np + bs - 1) / bs, bs, 0, st>>>(key, src.id, counts, cells, slot, idslot, np);
+    const int nt = cell_tiles(ncell);
+    if (out.shift == kCellTileLog2) {
+        const int bs = nt > 256 ? 256 : wave_block(k_scatter<true>, np);
+        k_scatter<true><<<(np + bs - 1) / bs, bs, 0, st>>>(key, src.id, counts, out, nt, slot, idslot, np);
+    } else {
+        const int bs = wave_block(k_scatter<false>, np);
+        k_scatter<false><<<(np + bs - 1) / bs, bs, 0, st>>>(key, src.id, counts, out, nt, slot, idslot, np);
+    }
+    const CellList cells{out.local, out.base, out.shift};
     if (dim == 2) {
         const int b = wave_block(k_gather<2, Real>, np);
         k_gather<2, Real><<<(np + b - 1) / b, b, 0, st>>>(cells, slot, idslot, src, dst, np);
@@ -1073,9 +1115,9 @@ k_cell_scan_batched(const BatchBed *__restrict__ beds, const int2 *__restrict__ 
         const int nt = (b.ncell + 1 + (1 << b.cl_shift) - 1) >> b.cl_shift;
         __syncthreads();   // the previous entry's users of the shared words are done
         if (b.cl_shift == kCellTileLog2Large)
-            cell_scan_tile<16>(b.counts, out, b.ncell + 1, e.tile, nt, warp_tot, total, last);
+            cell_scan_tile<16, true>(b.counts, out, b.ncell + 1, e.tile, nt, warp_tot, total, last);
         else
-            cell_scan_tile<4>(b.counts, out, b.ncell + 1, e.tile, nt, warp_tot, total, last);
+            cell_scan_tile<4, true>(b.counts, out, b.ncell + 1, e.tile, nt, warp_tot, total, last);
     }
 }
 
@@ -1091,7 +1133,7 @@ k_scatter_batched(const BatchBed *__restrict__ beds, const int2 *__restrict__ wo
         const int k = e.tile * kBatchTile + (int)threadIdx.x;
         if (k >= b.np) continue;
         const int nb = 1 - e.a;
-        scatter_one(b.key, b.part[e.a].id, b.counts, CellList{b.cl_local[nb], b.cl_base[nb], b.cl_shift}, b.slot,
+        scatter_one(b.key, b.part[e.a].id, b.counts, b.cl_local[nb], b.cl_base[nb], b.cl_shift, b.slot,
                     b.idslot, k);
     }
 }
@@ -1196,9 +1238,9 @@ template void launch_spins_to_host_order<3, double>(Particles<double>, int, doub
 template void launch_spins_to_host_order<1, float>(Particles<float>, int, double, double *, cudaStream_t);
 template void launch_spins_to_host_order<3, float>(Particles<float>, int, double, double *, cudaStream_t);
 
-template void launch_place<double>(int, const int *, int *, CellList, int2 *, int *,
+template void launch_place<double>(int, const int *, int *, CellListOut, int, int2 *, int *,
                                    Particles<double>, Particles<double>, int, cudaStream_t);
-template void launch_place<float>(int, const int *, int *, CellList, int2 *, int *,
+template void launch_place<float>(int, const int *, int *, CellListOut, int, int2 *, int *,
                                   Particles<float>, Particles<float>, int, cudaStream_t);
 
 }  // namespace lbdpsk

@@ -348,10 +348,19 @@ k_contacts_binned(StepParams<Real> p, Particles<Real> parts, CellList cells, Rea
     const Real d2_hi = (Real)p.d2 + contact_band<Real>();
     Real F[3] = {Real(0), Real(0), Real(0)}, T[3] = {Real(0), Real(0), Real(0)};
 
-    for (int s = first; s < end;) {
+    // The thin top of a 3D bed spreads a block over many rows, a run for each and
+    // some 15 us a run: there gridDim.y blocks share the runs.  The 16 x 16 x 32
+    // bed's launch grew from 120 to 366 us as its top loosened with one, to 177
+    // with four and 153 with eight; spare blocks leave at once (a steady launch:
+    // 110.5 us with one, 109 with eight).
+    if (blockIdx.y > 0 && p.by_row(__ldg(parts.cell + end - 1)) - p.by_row(__ldg(parts.cell + first)) < (int)blockIdx.y)
+        return;
+    bool taken = false;   // the thread's particle was in one of this block's runs
+    for (int s = first, e, turn = 0; s < end; s = e, turn = turn + 1 == (int)gridDim.y ? 0 : turn + 1) {
         // the run [s, e): the particles left in the row of slot s (at most kRowCells cells)
         const int c0 = __ldg(parts.cell + s), xa = c0 - p.by_row(c0) * p.n[0], row = c0 - xa;
-        const int e = min(end, cells.begin(row + min(p.n[0], xa + kRowCells)));
+        e = min(end, cells.begin(row + min(p.n[0], xa + kRowCells)));
+        if (turn != (int)blockIdx.y) continue;
         const int xb = __ldg(parts.cell + e - 1) - row;
         const int ncx = xb - xa + 1;
         int ri[3];
@@ -361,6 +370,7 @@ k_contacts_binned(StepParams<Real> p, Particles<Real> parts, CellList cells, Rea
         while (m > 1 && (ncx * m + 2) * (m + 2) * (D == 3 ? m + 2 : 1) > kBinMax) --m;
         const int nxs = ncx * m + 2, nys = m + 2, nb = nxs * nys * (D == 3 ? nys : 1);
         const bool mine = i >= s && i < e;
+        taken = taken || mine;
         // subcell of an in-cell offset
         auto sub = [&](Real o) { return min((int)(o * (Real)m), m - 1); };
         const int bx = (idx[0] - xa) * m + sub(oi[0]), by = sub(oi[1]), bz = D == 3 ? sub(oi[2]) : 0;
@@ -617,10 +627,9 @@ k_contacts_binned(StepParams<Real> p, Particles<Real> parts, CellList cells, Rea
                 __syncthreads();
             }
         }
-        s = e;
         __syncthreads();
     }
-    if (i < np) finish_contacts<D, Real, FRIC>(p, parts, i, idx, per, vi, wi, F, T, diag_fc, np);
+    if (taken) finish_contacts<D, Real, FRIC>(p, parts, i, idx, per, vi, wi, F, T, diag_fc, np);
 }
 
 // Mean particles per cell from which the binned kernel is taken.  Both sides on
@@ -643,7 +652,8 @@ static void launch_contacts_fric(const StepParams<Real> &p, Particles<Real> part
         // a refusal shows as the launch's error
         cudaFuncSetAttribute(k_contacts_binned<D, Real, FRIC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
-        k_contacts_binned<D, Real, FRIC><<<(np + kBinThreads - 1) / kBinThreads, kBinThreads, smem, st>>>(
+        const dim3 grid((np + kBinThreads - 1) / kBinThreads, D == 3 ? 8 : 1);
+        k_contacts_binned<D, Real, FRIC><<<grid, kBinThreads, smem, st>>>(
             p, parts, cells, diag_fc, np);
     } else {
         const int b = wave_block(k_contacts<D, Real, FRIC>, np);

@@ -45,6 +45,18 @@ def _bed(name):
         x = (np.arange(0, 400, 3) + 0.5) * w.h
         pos = np.concatenate([w.pos, np.stack([x, np.full_like(x, 4.5 * w.h)], axis=1)])
         return w.with_(bc=(P, P, N, N, P, P), pos=pos, vel=np.concatenate([w.vel, np.zeros((len(x), 2))]))
+    if name == "2d-thin-top":    # a crowded layer under rows of a few particles each
+        w = W.packed_bed(n=(8, 60), fill_rows=24, n_particles=2400)
+        y, x = np.meshgrid(np.arange(26, 60), np.arange(1, 8, 3), indexing="ij")
+        pos = np.stack([(x.ravel() + 0.5) * w.h, (y.ravel() + 0.5) * w.h], axis=1)
+        pos = np.concatenate([pos, pos + [0.18 * w.h, 0.0]])   # pairs in contact
+        return w.with_(pos=np.concatenate([w.pos, pos]), vel=np.concatenate([w.vel, np.zeros_like(pos)]))
+    if name == "3d-thin-top":    # the same in 3D: more runs than blocks that share them
+        w = W.packed_bed(dim=3, n=(6, 7, 12), fill_rows=3, n_particles=int(7.5 * 504))
+        z, y, x = np.meshgrid(np.arange(4, 12), np.arange(7), np.arange(0, 6, 2), indexing="ij")
+        pos = (np.stack([x.ravel(), y.ravel(), z.ravel()], axis=1) + 0.4) * w.h
+        pos = np.concatenate([pos, pos + [0.0, 0.18 * w.h, 0.0]])
+        return w.with_(pos=np.concatenate([w.pos, pos]), vel=np.concatenate([w.vel, np.zeros_like(pos)]))
     if name == "2d-pressed":     # more pairs than a list and more candidates than a chunk hold
         return W.packed_bed(n=(6, 10), fill_rows=5, n_particles=6 * 5 * 88, gap=0.3)
     if name == "3d-below":
@@ -58,8 +70,8 @@ def _bed(name):
 
 @pytest.mark.parametrize("name,storage", [
     ("2d-below", W.STORE_F32), ("2d-above", W.STORE_F32), ("2d-above", W.STORE_F64),
-    ("2d-periodic", W.STORE_F32), ("2d-long-run", W.STORE_F32), ("2d-pressed", W.STORE_F64),
-    ("3d-below", W.STORE_F32), ("3d-above", W.STORE_F32), ("3d-pressed", W.STORE_F64)])
+    ("2d-periodic", W.STORE_F32), ("2d-long-run", W.STORE_F32), ("2d-thin-top", W.STORE_F32), ("2d-pressed", W.STORE_F64),
+    ("3d-below", W.STORE_F32), ("3d-above", W.STORE_F32), ("3d-thin-top", W.STORE_F32), ("3d-pressed", W.STORE_F64)])
 @pytest.mark.parametrize("friction", [False, True])
 def test_contact_kernels_against_oracle(name, storage, friction):
     from paper_1303_2653_gb300 import lbdps as L

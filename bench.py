@@ -1004,8 +1004,8 @@ def dem_main(args):
             "roofline_contacts": {"bound": "hbm", "achieved": ach, "peak": peak,
                                   "peak_kind": peak_kind, "unit": "GB/s", "frac": ach / peak,
                                   "bytes_per_launch": nb,
-                                  "limiter": "instruction issue: the walk over the candidates "
-                                             "of the cells within reach"},
+                                  "limiter": "instruction issue and block barriers: the search "
+                                             "of the binned candidates"},
             "health": s["health"], "clocks": clk}
     print(json.dumps(line), flush=True)
     bed.close()

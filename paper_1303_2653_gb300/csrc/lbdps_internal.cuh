@@ -480,12 +480,15 @@ void launch_snapshot(const unsigned *health, const unsigned long long *solids_ou
 // (launch_gas_moments, or a collision with gas_partials); parts = the
 // particles of that state in sorted (cell) order; bed = the diagnostic
 // fields or null; ticket must be zero on entry and is zero again on exit.
+// record (or null): out points at record 0 of an array of kStatOut doubles each,
+// the result goes to record *record, which is then counted up (a captured
+// launch that runs again writes the next record).
 template <class L, class Real>
 void launch_reduce_all(int ncell, const double *gas, long long ngas, Particles<Real> parts, double mp,
                        int np, const Real *eps_tab, int ntab, const Fields<Real> *bed,
                        double *partials, unsigned *ticket,
                        const unsigned *health, const unsigned long long *solids_out, double *out,
-                       unsigned *health_live, int packed_limit, cudaStream_t st);
+                       unsigned *health_live, int packed_limit, int *record, cudaStream_t st);
 
 int reduce_block_count(int n);
 

@@ -62,7 +62,7 @@ k_reduce_all(int ncell, const double *__restrict__ gas, long long ngas, Particle
              double mp, int np, const Real *__restrict__ eps_tab, int ntab,
              Fields<Real> fld, double *partials, unsigned *ticket, const unsigned *health,
              const unsigned long long *solids_out, double *out, unsigned *health_live,
-             int packed_limit)
+             int packed_limit, int *record)
 {
     constexpr int D = L::D;
     Acc<Real> acc[kStatValues];
@@ -144,6 +144,8 @@ k_reduce_all(int ncell, const double *__restrict__ gas, long long ngas, Particle
     __syncthreads();
     if (!last) return;
     __threadfence();
+    // the place of this record where the launch counts them itself
+    if (record) out += (size_t)__ldcg(record) * kStatOut;
     // the last block: warp w adds values w, w + 8, ...; its lane l adds the
     // partials of blocks l, l + 32, ... in that order (independent loads,
     // issued eight at a time), then the warp adds its lanes in a fixed order
@@ -162,6 +164,10 @@ k_reduce_all(int ncell, const double *__restrict__ gas, long long ngas, Particle
         raw[kStatValues + 1] = *solids_out;
         *ticket = 0u;
     }
+    if (record) {
+        __syncthreads();   // every thread has its place
+        if (threadIdx.x == 0) ++*record;
+    }
 }
 
 template <class L, class Real>
@@ -169,7 +175,7 @@ void launch_reduce_all(int ncell, const double *gas, long long ngas, Particles<R
                        int np, const Real *eps_tab, int ntab,
                        const Fields<Real> *bed, double *partials, unsigned *ticket,
                        const unsigned *health, const unsigned long long *solids_out, double *out,
-                       unsigned *health_live, int packed_limit, cudaStream_t st)
+                       unsigned *health_live, int packed_limit, int *record, cudaStream_t st)
 {
     // the cells are walked only for the diagnostics
     long long n = bed ? (ncell > np ? ncell : np) : np;
@@ -179,11 +185,11 @@ void launch_reduce_all(int ncell, const double *gas, long long ngas, Particles<R
     if (bed)
         k_reduce_all<L, Real, true><<<(int)nb, kRedThreads, 0, st>>>(
             ncell, gas, ngas, parts, mp, np, eps_tab, ntab, *bed, partials, ticket, health,
-            solids_out, out, health_live, packed_limit);
+            solids_out, out, health_live, packed_limit, record);
     else
         k_reduce_all<L, Real, false><<<(int)nb, kRedThreads, 0, st>>>(
             ncell, gas, ngas, parts, mp, np, eps_tab, ntab, Fields<Real>{}, partials, ticket,
-            health, solids_out, out, health_live, packed_limit);
+            health, solids_out, out, health_live, packed_limit, record);
 }
 
 // The health word and the outlet count at the end of a step, for the
@@ -208,7 +214,7 @@ void launch_snapshot(const unsigned *health, const unsigned long long *solids_ou
                                           int, const R *, int, const Fields<R> *,                    \
                                           double *, unsigned *, const unsigned *,                    \
                                           const unsigned long long *, double *, unsigned *, int,     \
-                                          cudaStream_t);
+                                          int *, cudaStream_t);
 LBDPS_INST_RED(D2Q9, double)
 LBDPS_INST_RED(D2Q9, float)
 LBDPS_INST_RED(D3Q19, double)

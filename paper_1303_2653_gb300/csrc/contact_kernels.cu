@@ -352,9 +352,13 @@ k_contacts_binned(StepParams<Real> p, Particles<Real> parts, CellList cells, Rea
     // some 15 us a run: there gridDim.y blocks share the runs.  The 16 x 16 x 32
     // bed's launch grew from 120 to 366 us as its top loosened with one, to 177
     // with four and 153 with eight; spare blocks leave at once (a steady launch:
-    // 110.5 us with one, 109 with eight).
-    if (blockIdx.y > 0 && p.by_row(__ldg(parts.cell + end - 1)) - p.by_row(__ldg(parts.cell + first)) < (int)blockIdx.y)
-        return;
+    // 110.5 us with one, 109 with eight).  A row of n[0] cells holds at most
+    // ceil(n[0] / kRowCells) runs, each of which starts kRowCells cells or more
+    // after the one before.
+    if (blockIdx.y > 0) {
+        const int rows = p.by_row(__ldg(parts.cell + end - 1)) - p.by_row(__ldg(parts.cell + first)) + 1;
+        if ((long long)rows * ((p.n[0] + kRowCells - 1) / kRowCells) <= (int)blockIdx.y) return;
+    }
     bool taken = false;   // the thread's particle was in one of this block's runs
     for (int s = first, e, turn = 0; s < end; s = e, turn = turn + 1 == (int)gridDim.y ? 0 : turn + 1) {
         // the run [s, e): the particles left in the row of slot s (at most kRowCells cells)

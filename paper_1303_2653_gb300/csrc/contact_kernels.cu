@@ -225,15 +225,13 @@ __device__ __forceinline__ void finish_contacts(const StepParams<Real> &p,
     }
 }
 
-// One thread per particle (sparse beds): each walks the cells within its own
-// reach.  FRIC: soft spheres with friction (spins read from parts.w, the new
-// spins written to p.spin_out).
+// The contacts of particle i by a walk over the cells within its own reach.
+// FRIC: soft spheres with friction (spins read from parts.w, the new spins
+// written to p.spin_out).
 template <int D, class Real, bool FRIC>
-__global__ void __launch_bounds__(256, ContactOccupancy<D, Real, FRIC>::value)
-k_contacts(StepParams<Real> p, Particles<Real> parts, CellList cells, Real *diag_fc, int np)
+__device__ __forceinline__ void walk_contacts(const StepParams<Real> &p, const Particles<Real> &parts,
+                                              const CellList &cells, Real *diag_fc, int np, int i)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= np) return;
     int idx[3];
     cell_coords<D, Real>(p, __ldg(parts.cell + i), idx);
     float oi[3] = {0.f, 0.f, 0.f};
@@ -276,6 +274,16 @@ k_contacts(StepParams<Real> p, Particles<Real> parts, CellList cells, Real *diag
     finish_contacts<D, Real, FRIC>(p, parts, i, idx, per, vi, wi, F, T, diag_fc, np);
 }
 
+// One thread per particle (sparse beds).
+template <int D, class Real, bool FRIC>
+__global__ void __launch_bounds__(256, ContactOccupancy<D, Real, FRIC>::value)
+k_contacts(StepParams<Real> p, Particles<Real> parts, CellList cells, Real *diag_fc, int np)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= np) return;
+    walk_contacts<D, Real, FRIC>(p, parts, cells, diag_fc, np, i);
+}
+
 // Crowded beds: one block per kBinThreads consecutive sorted particles, a
 // thread each.  They lie in a few runs of cells along x; for each run the block
 // reads every particle of the rows around it once, keeps those within reach of
@@ -290,13 +298,20 @@ k_contacts(StepParams<Real> p, Particles<Real> parts, CellList cells, Real *diag
 // different sets of cells, so a warp runs as long as its slowest lane with a
 // third of its lanes busy, at 22 (2D, 11 particles per cell) to 230 (3D, 84 per
 // cell) candidates per particle, and evaluates each lane's few contacts alone.
-// Block and shared-memory shape.
+// Block and shared-memory shape; blocks per SM in FP32 without and with friction
+// (2D: 48 registers instead of 40 with spills, 99 -> 95 us on the bed of 256 x
+// 1024 cells; with friction the shared memory holds 9); blocks that share the
+// runs of a group of slots, and the runs that each of them takes at most (FP64:
+// a walk costs five times the time there, so it is left to more runs: rows of
+// 2 cells at 11 per cell 316 us with 8, 420 with 3, walk alone 486).
 template <int D> struct BinShape;
 template <> struct BinShape<2> {
-    static constexpr int threads = 128, cap = 384, bins = 384, hits = 8, blocks_f32 = 12;
+    static constexpr int threads = 128, cap = 384, bins = 384, hits = 8, blocks_f32 = 10, blocks_fric = 9;
+    static constexpr int share = 1, runs_f32 = 3, runs_f64 = 8;
 };
 template <> struct BinShape<3> {
-    static constexpr int threads = 256, cap = 1024, bins = 1024, hits = 12, blocks_f32 = 3;
+    static constexpr int threads = 256, cap = 1024, bins = 1024, hits = 12, blocks_f32 = 3, blocks_fric = 3;
+    static constexpr int share = 8, runs_f32 = 4, runs_f64 = 4;
 };
 
 // in-cell offsets (in 2D o[2] holds the y cell offset of the candidate's row
@@ -322,7 +337,8 @@ template <int D, class Real, bool FRIC> struct ContactBins {
 };
 
 template <int D, class Real, bool FRIC>
-__global__ void __launch_bounds__(BinShape<D>::threads, sizeof(Real) == 4 ? BinShape<D>::blocks_f32 : 1)
+__global__ void __launch_bounds__(BinShape<D>::threads, sizeof(Real) != 4 ? 1 : FRIC ? BinShape<D>::blocks_fric
+                                                                                : BinShape<D>::blocks_f32)
 k_contacts_binned(StepParams<Real> p, Particles<Real> parts, CellList cells, Real *diag_fc, int np)
 {
     extern __shared__ __align__(16) unsigned char bins_smem[];
@@ -357,23 +373,35 @@ k_contacts_binned(StepParams<Real> p, Particles<Real> parts, CellList cells, Rea
     const ContactReach<Real> reach(p);
     Real F[3] = {Real(0), Real(0), Real(0)}, T[3] = {Real(0), Real(0), Real(0)};
 
-    // The thin top of a 3D bed spreads a block over many rows, a run for each and
-    // some 15 us a run: there gridDim.y blocks share the runs.  The 16 x 16 x 32
-    // bed's launch grew from 120 to 366 us as its top loosened with one, to 177
-    // with four and 153 with eight; spare blocks leave at once (a steady launch:
-    // 110.5 us with one, 109 with eight).  A row of n[0] cells holds at most
-    // ceil(n[0] / kRowCells) runs, each of which starts kRowCells cells or more
-    // after the one before.
+    // The thin top of a bed spreads a block over many rows, a run for each, at
+    // 2-3 us a run in 2D and 5-15 in 3D.  In 3D gridDim.y blocks share the runs:
+    // the 16 x 16 x 32 bed's launch grew from 120 to 366 us as its top loosened
+    // with one, to 177 with four and 153 with eight; spare blocks leave at once (a
+    // steady launch: 110.5 us with one, 109 with eight).  A row of n[0] cells
+    // holds at most ceil(n[0] / kRowCells) runs, each of which starts kRowCells
+    // cells or more after the one before.
     if (blockIdx.y > 0) {
         const int rows = p.by_row(__ldg(parts.cell + end - 1)) - p.by_row(__ldg(parts.cell + first)) + 1;
         if ((long long)rows * ((p.n[0] + kRowCells - 1) / kRowCells) <= (int)blockIdx.y) return;
     }
+    // The slots past the first share * runs runs are walked a thread each, as in
+    // k_contacts: so few particles to a run have few candidates.  64 x 512 cells,
+    // the lower half at 11 per cell, one particle in each row above: 294 us with
+    // every run binned, 25.7 so (walk alone 33; at most 2, 4 and 8 runs: 25.7, 27.7
+    // and 36); 16 x 16 x 32, a third at 30 per cell, one in each row above, friction:
+    // 164 us, 47 so (walk alone 70; 64 runs 64).
+    constexpr int kRuns = BinShape<D>::share * (sizeof(Real) == 4 ? BinShape<D>::runs_f32 : BinShape<D>::runs_f64);
+    int rest = end;
     bool taken = false;   // the thread's particle was in one of this block's runs
-    for (int s = first, e, turn = 0; s < end; s = e, turn = turn + 1 == (int)gridDim.y ? 0 : turn + 1) {
+    for (int s = first, e, run = 0; s < end; s = e, ++run) {
+        if (run == kRuns) {
+            rest = s;
+            break;
+        }
         // the run [s, e): the particles left in the row of slot s (at most kRowCells cells)
         const int c0 = __ldg(parts.cell + s), xa = c0 - p.by_row(c0) * p.n[0], row = c0 - xa;
         e = min(end, cells.begin(row + min(p.n[0], xa + kRowCells)));
-        if (turn != (int)blockIdx.y) continue;
+        if (run % BinShape<D>::share != (int)blockIdx.y) continue;
         const int xb = __ldg(parts.cell + e - 1) - row;
         const int ncx = xb - xa + 1;
         int ri[3];
@@ -509,14 +537,14 @@ k_contacts_binned(StepParams<Real> p, Particles<Real> parts, CellList cells, Rea
                 }
                 if (lane == 31) t.warp_tot[warp] = inc;
                 __syncthreads();
-                int run = inc - sum;
+                int at = inc - sum;
 #pragma unroll
                 for (int w = 0; w < kBinThreads / 32; ++w)
-                    if (w < warp) run += t.warp_tot[w];
+                    if (w < warp) at += t.warp_tot[w];
 #pragma unroll
                 for (int k = 0; k < kPer; ++k) {
-                    if (lo + k < nb) t.start[lo + k] = run;
-                    run += v[k];
+                    if (lo + k < nb) t.start[lo + k] = at;
+                    at += v[k];
                 }
                 if (tid == 0) {
                     t.start[nb] = kept;
@@ -643,6 +671,7 @@ k_contacts_binned(StepParams<Real> p, Particles<Real> parts, CellList cells, Rea
         __syncthreads();
     }
     if (taken) finish_contacts<D, Real, FRIC>(p, parts, i, idx, per, vi, wi, F, T, diag_fc, np);
+    else if (blockIdx.y == 0 && i >= rest && i < np) walk_contacts<D, Real, FRIC>(p, parts, cells, diag_fc, np, i);
 }
 
 // Mean particles per cell from which the binned kernel is taken.  Both sides on
@@ -665,7 +694,7 @@ static void launch_contacts_fric(const StepParams<Real> &p, Particles<Real> part
         // a refusal shows as the launch's error
         cudaFuncSetAttribute(k_contacts_binned<D, Real, FRIC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
-        const dim3 grid((np + kBinThreads - 1) / kBinThreads, D == 3 ? 8 : 1);
+        const dim3 grid((np + kBinThreads - 1) / kBinThreads, BinShape<D>::share);
         k_contacts_binned<D, Real, FRIC><<<grid, kBinThreads, smem, st>>>(
             p, parts, cells, diag_fc, np);
     } else {

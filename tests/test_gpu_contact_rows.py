@@ -1,8 +1,10 @@
-"""GPU vs oracle: the binned soft-sphere contacts of a 3D bed whose rows are cut into several runs
-while the blocks of a group of slots share those runs.
+"""GPU vs oracle: the binned soft-sphere contacts of beds whose thin top spreads a block over many
+runs of cells.
 
-A run spans at most 111 cells.  Two steps, each from a common start-of-step state: what a slot keeps
-from the step before must not pass for its force or spin.  Bounds as in test_gpu_soft_spheres.py.
+In 3D a run spans at most 111 cells and the blocks of a group of slots share its runs; beyond 3 runs
+(2D) or 32 (3D) a block walks for the particles left.  Two steps, each from a common start-of-step
+state: what a slot keeps from the step before must not pass for its force or spin.  Bounds as in
+test_gpu_soft_spheres.py.
 """
 import os
 import sys
@@ -32,16 +34,44 @@ def _built():
         pytest.skip("no CUDA device")
 
 
-def _bed(nx, every, bc):
-    """Two crowded planes (9 particles per cell of the bed) under rows that hold a pair in contact in
-    every `every`-th cell, so that 256 slots lie in one row, in two, or in nine and more."""
-    n = (nx, 4, 7)
-    w = W.packed_bed(dim=3, n=n, fill_rows=2, n_particles=9 * nx * 28)
-    z, y, x = np.meshgrid(np.arange(3, 7), np.arange(4), np.arange(0, nx, every), indexing="ij")
-    pos = (np.stack([x.ravel(), y.ravel(), z.ravel()], axis=1) + 0.4) * w.h
-    pos = np.concatenate([pos, pos + [0.18 * w.h, 0.0, 0.0]])
-    vel = np.random.default_rng(nx).normal(0.0, 0.05, size=pos.shape)
-    return w.with_(bc=bc, pos=np.concatenate([w.pos, pos]), vel=np.concatenate([w.vel, vel]))
+def _top(w, rows, x):
+    """w with a pair in contact in the cells x of every row of cells in rows (their y, or y and z)."""
+    rows = np.asarray(rows).reshape(len(rows), -1)
+    pos = np.column_stack([np.tile(x, len(rows)), np.repeat(rows, len(x), axis=0)]) + 0.4
+    step = np.zeros(w.dim)
+    step[0] = 0.18
+    pos = np.concatenate([pos, pos + step]) * w.h
+    vel = np.random.default_rng(len(pos)).normal(0.0, 0.05, size=pos.shape)
+    return w.with_(pos=np.concatenate([w.pos, pos]), vel=np.concatenate([w.vel, vel]))
+
+
+def _rows(w, first):
+    """the rows of cells from level `first` of the vertical axis on"""
+    if w.dim == 2:
+        return np.arange(first, w.n[1])
+    z, y = np.meshgrid(np.arange(first, w.n[2]), np.arange(w.n[1]), indexing="ij")
+    return np.stack([y.ravel(), z.ravel()], axis=1)
+
+
+def _check(w, storage):
+    from paper_1303_2653_gb300 import lbdps as L
+    bed, ob = _pair(w, storage)
+    tol = 1e-11 if storage == W.STORE_F64 else 1e-5
+    for step in range(2):
+        if step:
+            ob.set_populations(bed.populations())
+            ob.set_particles(*bed.particles())
+            if w.dem_mu > 0:
+                ob.set_spin(bed.spin())
+        bed.step(1)
+        ob.step(1)
+        fg, fo = bed.particle_diag(L.PDIAG_FC), ob.particle_diag(O.P_FC)
+        assert np.abs(fg - fo).max() <= tol * np.abs(fo).max(), step
+        if w.dem_mu > 0:
+            so = ob.spin()
+            assert np.abs(bed.spin() - so).max() <= tol * np.abs(so).max(), step
+    assert bed.check_guards() == 0
+    bed.close()
 
 
 @pytest.mark.parametrize("nx,every", [(111, 8), (112, 1), (112, 3), (113, 2), (160, 1), (160, 8), (300, 1),
@@ -50,24 +80,22 @@ def _bed(nx, every, bc):
 @pytest.mark.parametrize("friction", [False, True])
 @pytest.mark.parametrize("bc", [(N,) * 6, (P, P, N, N, N, N)])
 def test_rows_of_several_runs(nx, every, storage, friction, bc):
-    from paper_1303_2653_gb300 import lbdps as L
-    w = _bed(nx, every, bc)
-    w = W.with_friction(w) if friction else w
-    assert len(w.pos) >= 8 * nx * 28   # the binned kernel
-    bed, ob = _pair(w, storage)
-    tol = 1e-11 if storage == W.STORE_F64 else 1e-5
-    for step in range(2):
-        if step:
-            ob.set_populations(bed.populations())
-            ob.set_particles(*bed.particles())
-            if friction:
-                ob.set_spin(bed.spin())
-        bed.step(1)
-        ob.step(1)
-        fg, fo = bed.particle_diag(L.PDIAG_FC), ob.particle_diag(O.P_FC)
-        assert np.abs(fg - fo).max() <= tol * np.abs(fo).max(), step
-        if friction:
-            so = ob.spin()
-            assert np.abs(bed.spin() - so).max() <= tol * np.abs(so).max(), step
-    assert bed.check_guards() == 0
-    bed.close()
+    # two crowded planes (9 particles per cell of the bed) under rows that hold a pair in every
+    # `every`-th cell, so that 256 slots lie in one row, in two, or in nine and more
+    w = W.packed_bed(dim=3, n=(nx, 4, 7), fill_rows=2, n_particles=9 * nx * 28)
+    w = _top(w, _rows(w, 3), np.arange(0, nx, every)).with_(bc=bc)
+    _check(W.with_friction(w) if friction else w, storage)
+
+
+# pairs in a row of the top: runs of a block far beyond the limit, at it and just past it, below it
+@pytest.mark.parametrize("dim,pairs", [(2, 1), (2, 8), (2, 14), (2, 16), (3, 1), (3, 3), (3, 4), (3, 9)])
+@pytest.mark.parametrize("storage", [W.STORE_F64, W.STORE_F32])
+@pytest.mark.parametrize("friction", [False, True])
+def test_thin_tops(dim, pairs, storage, friction):
+    if dim == 2:
+        w = W.packed_bed(n=(16, 60), fill_rows=24, n_particles=15 * 384, gap=0.8)
+        w = _top(w, _rows(w, 25), np.arange(16)[::-1][:pairs])
+    else:
+        w = W.packed_bed(dim=3, n=(16, 6, 16), fill_rows=4, n_particles=39 * 384)
+        w = _top(w, _rows(w, 5), np.arange(16)[::-1][:pairs])
+    _check(W.with_friction(w) if friction else w, storage)

@@ -674,21 +674,43 @@ k_contacts_binned(StepParams<Real> p, Particles<Real> parts, CellList cells, Rea
     else if (blockIdx.y == 0 && i >= rest && i < np) walk_contacts<D, Real, FRIC>(p, parts, cells, diag_fc, np, i);
 }
 
-// Mean particles per cell from which the binned kernel is taken.  Both sides on
-// a GB300, particles spread evenly, d = 0.2 (us; 2D 256 x 1024, 3D 48 x 48 x 64):
-//     2D per cell     2          4          5.6 (lower half filled: 11)
-//     walk / binned   26 / 43    59 / 70    155 / 93
-//     3D per cell     2          4          16
-//     walk / binned   39 / 94    97 / 141   917 / 507
-// The bed of 256 x 1024 cells took 155 us per launch with the walk alone, the
-// 3D bed of 16 x 16 x 32 cells (42 per cell, friction) 660 us against 112.
-template <int D> constexpr int kBinOccupancy = D == 2 ? 5 : 8;
+// Whether the binned kernel is taken.  It pays by the particles per cell, and the
+// narrower the rows, the more runs a block has.  Both sides on a GB300, d = 0.2
+// (us; even: spread evenly, half: the lower half filled, particles per cell of
+// the whole bed), walk / binned:
+//     2D      even 5     even 5.5   even 7      even 9      half 5.6
+//     512^2   80 / 87    92 / 91    135 / 113   206 / 140   158 / 108
+//     256^2   29 / 32    33 / 34    45 / 40     63 / 49     51 / 38
+//     64^2    16 / 20    16 / 20    19 / 20     21 / 20     23 / 20
+//     2D rows of   16          12         10         8          6          4 cells
+//     even 8       41 / 42     42 / 47    42 / 47    41 / 53    42 / 65    41 / 68
+//     even 11      67 / 52     66 / 55    66 / 59    66 / 63    67 / 70    65 / 99
+//     half 5.6     51 / 40     51 / 42    52 / 45    53 / 48    51 / 52    51 / 72
+//     3D                 even 8      even 10    even 12    even 20    half 25, friction
+//     48 x 48 x 64       295 / 280
+//     20 x 20 x 40       46 / 50     66 / 55
+//     8 x 40 x 40        44 / 56                60 / 64    149 / 85   428 / 118
+//     4 x 40 x 40        29 / 46                35 / 52    83 / 62    247 / 72
+//     2 x 40 x 40        26 / 38                32 / 42    46 / 54    153 / 52
+// 2D: 5.5 per cell lies between the two fillings' own lines, and 66 per row holds
+// both.  3D: 8 per cell in wide beds, the more the narrower the rows.  In FP64 a
+// pair tested costs the walk more (the FP64 pipe) and the lines lie lower: 256 x
+// 256 even 5.1 288 / 175; rows of 4 cells, 2D, even 5.1 130 / 153 and 8 276 / 182;
+// of 2 cells even 8 271 / 279, 11 486 / 316; 3D rows of 1 cell even 12 91 / 107,
+// 20 137 / 123, of 2 cells even 8.1 104 / 97.
+template <int D, class Real> static bool bins_pay(long long np, long long ncell, long long n0)
+{
+    const long long rows = ncell / n0;
+    constexpr bool f32 = sizeof(Real) == 4;
+    if (D == 2) return 2 * np >= (f32 ? 11 : 10) * ncell && np >= (f32 ? 66 : 22) * rows;
+    return f32 ? np >= 8 * ncell + 20 * rows : np >= 8 * ncell && np >= 16 * rows;
+}
 
 template <int D, class Real, bool FRIC>
 static void launch_contacts_fric(const StepParams<Real> &p, Particles<Real> parts, CellList cells,
                                  Real *diag_fc, int np, cudaStream_t st)
 {
-    if ((long long)np >= (long long)kBinOccupancy<D> * p.ncell) {
+    if (bins_pay<D, Real>(np, p.ncell, p.n[0])) {
         constexpr size_t smem = sizeof(ContactBins<D, Real, FRIC>);
         constexpr int kBinThreads = BinShape<D>::threads;
         // a refusal shows as the launch's error

@@ -99,3 +99,31 @@ def test_thin_tops(dim, pairs, storage, friction):
         w = W.packed_bed(dim=3, n=(16, 6, 16), fill_rows=4, n_particles=39 * 384)
         w = _top(w, _rows(w, 5), np.arange(16)[::-1][:pairs])
     _check(W.with_friction(w) if friction else w, storage)
+
+
+# either side of the rule that takes the binned kernel, and forms of it that only crowded rows reach
+EDGES = [
+    # 2D: 5.5 per cell in FP32, 5 in FP64; 66 and 22 per row; runs over a whole row of periodic cells
+    ((64, 24), 8447, (N,) * 6), ((64, 24), 8448, (N,) * 6), ((64, 24), 7679, (N,) * 6), ((64, 24), 7680, (N,) * 6),
+    ((11, 60), 3959, (N,) * 6), ((11, 60), 3960, (N,) * 6), ((4, 60), 1319, (N,) * 6), ((4, 60), 1320, (N,) * 6),
+    ((3, 40), 120 * 23, (P,) * 6), ((13, 33), 429 * 7, (P, P, N, N, P, P)),
+    # 3D: 8 per cell and, in FP32, 20 per row more, in FP64 16 per row at least
+    ((24, 5, 9), 9539, (N,) * 6), ((24, 5, 9), 9540, (N,) * 6), ((24, 5, 9), 8639, (N,) * 6), ((24, 5, 9), 8640, (N,) * 6),
+    ((3, 6, 7), 1847, (N,) * 6), ((3, 6, 7), 1848, (N,) * 6), ((1, 6, 7), 671, (N,) * 6), ((1, 6, 7), 672, (N,) * 6),
+    ((3, 4, 5), 60 * 30, (P, P, P, P, N, N))]
+
+
+@pytest.mark.parametrize("n,particles,bc", EDGES)
+@pytest.mark.parametrize("storage", [W.STORE_F64, W.STORE_F32])
+@pytest.mark.parametrize("friction", [False, True])
+def test_either_side_of_the_rule(n, particles, bc, storage, friction):
+    w = W.packed_bed(dim=len(n), n=n, fill_rows=n[-1], n_particles=particles, gap=0.7).with_(bc=bc)
+    _check(W.with_friction(w) if friction else w, storage)
+
+
+@pytest.mark.parametrize("friction", [False, True])
+def test_long_sparse_rows_2d(friction):
+    # a row so sparse that its run is cut, above crowded ones
+    w = W.packed_bed(n=(400, 6), fill_rows=2, n_particles=13600, gap=0.8)
+    w = _top(w, [4, 5], np.arange(0, 400, 3)).with_(bc=(P, P, N, N, P, P))
+    _check(W.with_friction(w) if friction else w, W.STORE_F32)

@@ -454,7 +454,8 @@ template <class L, class Real, class S> struct EngineT : Engine {
         fld.rho = (Real *)get(sizeof(Real) * nc);
         fld.node4 = (typename Vec4<Real>::type *)get(sizeof(typename Vec4<Real>::type) * nc);
         fld.solg = D == 3 ? (Real *)get(sizeof(Real) * nc) : nullptr;
-        for (int a = 0; a < D; ++a) fld.fpg[a] = (Real *)get(sizeof(Real) * (D == 2 ? nc : np));
+        fld.fpg_by_cell = D == 2 || np >= nc;
+        for (int a = 0; a < D; ++a) fld.fpg[a] = (Real *)get(sizeof(Real) * (fld.fpg_by_cell ? nc : np));
         if (H->prm.diagnostics) {
             fld.tau_t = (Real *)get(sizeof(Real) * nc);
             fld.eps_g = (Real *)get(sizeof(Real) * nc);
@@ -919,7 +920,7 @@ template <class L, class Real, class S> struct EngineT : Engine {
         };
         add(LBDPS_FIELD_RHO, 1, rs, fld.rho, nullptr, nullptr, 1);
         add(LBDPS_FIELD_U, D, us, fld.u[0], fld.u[1], fld.u[2], 1);
-        add(LBDPS_FIELD_FPG, D, fs, fld.fpg[0], fld.fpg[1], fld.fpg[2], D == 2 ? 1 : 0);
+        add(LBDPS_FIELD_FPG, D, fs, fld.fpg[0], fld.fpg[1], fld.fpg[2], fld.fpg_by_cell ? 1 : 0);
         add(LBDPS_FIELD_BETA, 1, bs, node + 3, nullptr, nullptr, 4);
         add(LBDPS_FIELD_VS, D, us, fld.vs[0], fld.vs[1], fld.vs[2], 1);
         if (mask & LBDPS_FIELD_NTOT) x.counts = fld.ntot;

@@ -273,15 +273,17 @@ __host__ __device__ inline void cell_voidage(int dim, double r, double vp, int n
 // where a bed holds 0.06 particles per cell, it is kept for the occupied cells
 // alone, at the sorted slot of the cell's first particle in the step's input
 // list: 48 instead of 805 MB written per step of the 256 x 256 x 1024 riser
-// (collision 2,090 -> 1,966 us, drag 620 -> 576).  In 2D (0.4 and more per cell)
-// that saves little, and the slot lengthens the drag's chain of loads (75 x 193:
-// 22.2 -> 23.4 us a step), so it stays per cell.
+// (collision 2,090 -> 1,966 us, drag 620 -> 576).  A 3D bed of at least a particle
+// per cell keeps it per cell (fpg_by_cell), where a slot each would take more
+// memory.  In 2D (0.4 and more per cell) the slots save little and lengthen the
+// drag's chain of loads (75 x 193: 22.2 -> 23.4 us a step): always per cell.
 template <class Real> struct Fields {
     Real *rho, *fpg[3];                                 // node outputs of the collision
     typename Vec4<Real>::type *node4;
     Real *solg;                                         // 3D only (null in 2D)
     Real *vs[3], *tau_t, *u[3], *eps_g;                 // diagnostics (may be null)
     int *ntot;                                          // diagnostics (may be null)
+    bool fpg_by_cell;
 };
 
 // Particle arrays in cell-sorted order.  Besides the FP64 centre P and the

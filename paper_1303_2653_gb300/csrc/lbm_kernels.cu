@@ -450,7 +450,7 @@ __device__ __forceinline__ void collide_stream_cell(const StepParams<Real> &p, c
 #pragma unroll
     for (int a = 0; a < D; ++a) {
         const Real q = og * (rho * u[a] + rho * vs[a] - Real(2) * m[a]);
-        if (D == 2) fld.fpg[a][x] = q;
+        if (D == 2 || fld.fpg_by_cell) fld.fpg[a][x] = q;
         else if (n > 0) fld.fpg[a][s0] = q;   // see Fields
         ua[a] = u[a] * inv_div;
         const Real sl = ua[a] - vs[a];

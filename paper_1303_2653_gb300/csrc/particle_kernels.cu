@@ -300,7 +300,7 @@ __device__ __forceinline__ void drag_step_particle(const StepParams<Real> &p,
         s0 = cells.begin(c);
         s1 = cells.begin(c + 1);
 #pragma unroll
-        for (int a = 0; a < D; ++a) fpg[a] = __ldg(fld.fpg[a] + (D == 2 ? c : s0));
+        for (int a = 0; a < D; ++a) fpg[a] = __ldg(fld.fpg[a] + (D == 2 || fld.fpg_by_cell ? c : s0));
         cell_coords<D, Real>(p, c, idx);
         drag_pre_one<D, Real>(p, parts, fld, idx, o0, v0, fp, gp);
 #pragma unroll

@@ -303,7 +303,8 @@ k_contacts(StepParams<Real> p, Particles<Real> parts, CellList cells, Real *diag
 // 1024 cells; with friction the shared memory holds 9); blocks that share the
 // runs of a group of slots, and the runs that each of them takes at most (FP64:
 // a walk costs five times the time there, so it is left to more runs: rows of
-// 2 cells at 11 per cell 316 us with 8, 420 with 3, walk alone 486).
+// 2 cells at 11 per cell 277 us with 8, 420 with 3, all runs binned 316, walk
+// alone 486).
 template <int D> struct BinShape;
 template <> struct BinShape<2> {
     static constexpr int threads = 128, cap = 384, bins = 384, hits = 8, blocks_f32 = 10, blocks_fric = 9;

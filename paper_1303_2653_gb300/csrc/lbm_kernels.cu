@@ -109,7 +109,7 @@ void launch_build_tables(int dim, double tau, double r, double vp, double d, dou
 //                       + wg Omega^s_i + Guo source
 //   Eq. 25       F_p->g = wg (rho u + rho v_s - 2 m)  (sum_i c_i Omega^s_i in closed form)
 //   Eq. 19       node beta from |u/eps - v_s|
-//   Eq. 2        push streaming; half-way bounce-back (moving wall) on walls,
+//   Eq. 2        pull streaming from x - c_i; half-way bounce-back (moving wall) on walls,
 //                inlet/outlet incoming populations at feq(1, u_in | u)
 // All arithmetic on deviations f_i - w_i so that FP32 keeps the small
 // velocity moments accurate.
@@ -145,6 +145,8 @@ __device__ __forceinline__ double sqrt_pos(double x) { return sqrt(x); }
 // sums 64 (8 blocks: 128 x 128 x 512 BF16 294 us against 302); FP64 needs 114 (4
 // blocks: 512 x 2048 with LES 880 us against 913 with 8 and spills).
 constexpr int kCollideThreads = 128;
+// SMs that the lines in collide_shape were measured on: a tuning constant, not
+// the current device's count (any value gives the same results)
 constexpr int kSms = 152;
 template <class L, class Real, bool LES> struct K2Occupancy { static constexpr int value = 4; };
 #ifndef LBDPS_K2_BLOCKS_D2Q9_F32

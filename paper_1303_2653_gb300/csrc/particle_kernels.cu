@@ -597,9 +597,11 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *warp_tot, int *t
 // ---------------------------------------------------------------------------
 // One-launch scan of counts[0..ncell] into a two-level cell list.  Each block
 // scans one tile of 4,096 (or 16,384) counts, ITEMS consecutive counts per
-// thread in 16-byte loads and stores, and writes its total; the block that
-// finishes last (ticket counter, nothing waits) scans the tile totals and
-// resets the ticket for the next launch.
+// thread in 16-byte loads and stores, and writes its total.  The tile totals are
+// scanned (a) in the larger tiles and in batches by the block that finishes last
+// (ticket counter, nothing waits), which resets the ticket for the next launch,
+// (b) in a single bed's tiles of 4,096 by the scatter that follows: out.base holds
+// an older list until launch_place has run, and nothing may read the list before.
 // ---------------------------------------------------------------------------
 constexpr int kCellScanThreads = 1024;
 
@@ -812,7 +814,7 @@ template <class Real>
 void launch_place(int dim, const int *key, int *counts, CellListOut out, int ncell, int2 *slot,
                   int *idslot, Particles<Real> src, Particles<Real> dst, int np, cudaStream_t st)
 {
-    if (np == 0) return;
+    if (np == 0) return;   // out.base is not written: a bed without particles clears its list
     const int nt = cell_tiles(ncell);
     if (out.shift == kCellTileLog2) {
         const int bs = nt > 256 ? 256 : wave_block(k_scatter<true>, np);

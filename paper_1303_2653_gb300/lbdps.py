@@ -327,6 +327,8 @@ class Bed:
     # -- data -----------------------------------------------------------------
     def fields(self, mask: int = FIELD_RHO | FIELD_UACT | FIELD_FPG | FIELD_BETA,
                units: int = UNITS_LATTICE) -> Dict[str, np.ndarray]:
+        """Node fields by name, (cells,) or (cells, dim).  They are parts of one array:
+        copy a field that is to be kept without the others read with it."""
         sizes = []
         for bit, name in enumerate(FIELD_NAMES):
             if mask & (1 << bit):

@@ -212,8 +212,8 @@ def drag_step_bytes(w, storage):
 
 def rescale_force_saved(w, storage):
     """Bytes of the F_p->g node field that a 3D launch neither writes (the
-    collision) nor reads (the drag): the library keeps that force for occupied
-    cells only, counted here as one cell per particle."""
+    collision) nor reads (the drag): below a particle per cell the library keeps
+    that force for occupied cells only, counted here as one cell per particle."""
     if w.dim == 2:
         return 0
     return max(w.ncell - w.n_particles, 0) * w.dim * (8 if storage == "f64" else 4)
@@ -555,7 +555,11 @@ def measure_bed(L, torch, w, args, dist, world, peak, peak_kind, with_e2e=True):
                 acc[k] = acc.get(k, 0.0) + v
     per_kernel_ms = {k: v / prof_steps for k, v in acc.items()}
     alg_bytes, per_cell, per_particle = collide_stream_bytes(w, args.storage)
-    alg_bytes -= rescale_force_saved(w, args.storage)
+    saved = rescale_force_saved(w, args.storage)
+    alg_bytes -= saved
+    if saved:   # that force moves with the particles instead of the cells
+        force = w.dim * (8 if args.storage == "f64" else 4)
+        per_cell, per_particle = per_cell - force, per_particle + force
     cs_ms = per_kernel_ms["collide_stream"]
     achieved = alg_bytes / (cs_ms / 1e3) / 1e9
     traffic = profiled_traffic(w.name.split("-")[0] + "_" + "x".join(str(v) for v in w.n))
@@ -567,11 +571,11 @@ def measure_bed(L, torch, w, args, dist, world, peak, peak_kind, with_e2e=True):
     # the drag kernel against the same peak (in 3D the second largest share of
     # the step; in 2D about as long as collide_stream and bound by the
     # latency of dependent loads, not by bytes)
-    drag_bytes = drag_step_bytes(w, args.storage)[0] - rescale_force_saved(w, args.storage)
+    drag_bytes = drag_step_bytes(w, args.storage)[0] - saved
     roofline["drag"] = kernel_roofline(drag_bytes,
                                        per_kernel_ms.get("drag", 0.0), peak)
     ms_step = total_ms / args.steps
-    ws_bytes = whole_step_bytes(w, args.storage)
+    ws_bytes = whole_step_bytes(w, args.storage) - saved
     whole_step = {"algorithmic_bytes": ws_bytes, "ideal_ms": ws_bytes / (peak * 1e9) * 1e3,
                   "achieved": ws_bytes / (ms_step / 1e3) / 1e9,
                   "frac": ws_bytes / (ms_step / 1e3) / 1e9 / peak, "unit": "GB/s"}

@@ -312,7 +312,7 @@ template <> struct BinShape<2> {
 };
 template <> struct BinShape<3> {
     static constexpr int threads = 256, cap = 1024, bins = 1024, hits = 12, blocks_f32 = 3, blocks_fric = 3;
-    static constexpr int share = 8, runs_f32 = 4, runs_f64 = 4;
+    static constexpr int share = 8, runs_f32 = 6, runs_f64 = 6;
 };
 
 // in-cell offsets (in 2D o[2] holds the y cell offset of the candidate's row
@@ -390,7 +390,8 @@ k_contacts_binned(StepParams<Real> p, Particles<Real> parts, CellList cells, Rea
     // the lower half at 11 per cell, one particle in each row above: 294 us with
     // every run binned, 25.7 so (walk alone 33; at most 2, 4 and 8 runs: 25.7, 27.7
     // and 36); 16 x 16 x 32, a third at 30 per cell, one in each row above, friction:
-    // 164 us, 47 so (walk alone 70; 64 runs 64).
+    // 164 us, 54 so (walk alone 70; at most 32 and 64 runs: 46 and 64; but 32 cost
+    // 3 x 40 x 40 cells, half filled at 50, 119 us a step against 111).
     constexpr int kRuns = BinShape<D>::share * (sizeof(Real) == 4 ? BinShape<D>::runs_f32 : BinShape<D>::runs_f64);
     int rest = end;
     bool taken = false;   // the thread's particle was in one of this block's runs

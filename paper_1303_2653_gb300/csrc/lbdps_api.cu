@@ -903,6 +903,7 @@ template <class L, class Real, class S> struct EngineT : Engine {
         FieldExport<Real> x{};
         x.cells = cells(1 - H->parity);   // the input of the last step
         x.np = H->np;
+        x.fpg_by_cell = fld.fpg_by_cell;
         x.rho = fld.rho;
         x.node4 = fld.node4;
         auto add = [&](int bit, int count, double scale, const Real *a0, const Real *a1, const Real *a2,
@@ -920,7 +921,7 @@ template <class L, class Real, class S> struct EngineT : Engine {
         };
         add(LBDPS_FIELD_RHO, 1, rs, fld.rho, nullptr, nullptr, 1);
         add(LBDPS_FIELD_U, D, us, fld.u[0], fld.u[1], fld.u[2], 1);
-        add(LBDPS_FIELD_FPG, D, fs, fld.fpg[0], fld.fpg[1], fld.fpg[2], fld.fpg_by_cell ? 1 : 0);
+        add(LBDPS_FIELD_FPG, D, fs, fld.fpg[0], fld.fpg[1], fld.fpg[2], D == 2 ? 1 : 0);
         add(LBDPS_FIELD_BETA, 1, bs, node + 3, nullptr, nullptr, 4);
         add(LBDPS_FIELD_VS, D, us, fld.vs[0], fld.vs[1], fld.vs[2], 1);
         if (mask & LBDPS_FIELD_NTOT) x.counts = fld.ntot;

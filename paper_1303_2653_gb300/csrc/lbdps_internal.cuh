@@ -383,7 +383,7 @@ void launch_import_populations(const PopLayout &lay, int ncell, const double *in
 // Node fields exported one after the other: field i holds values f[i].first
 // on, count per cell (interleaved), component a of cell c read at
 // src[a][c * stride] and multiplied by scale.  src[0] null: the particle counts;
-// stride 0: kept per occupied cell (Fields::fpg), the list of that step in cells.
+// stride 0: kept for occupied cells (Fields::fpg), the list of that step in cells.
 template <class Real> struct FieldExport {
     struct {
         long long first;
@@ -392,6 +392,7 @@ template <class Real> struct FieldExport {
         const Real *src[3];
     } f[9];
     int nfield;
+    bool fpg_by_cell;
     long long total;
     const int *counts;
     CellList cells;

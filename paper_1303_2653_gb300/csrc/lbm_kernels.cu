@@ -452,8 +452,8 @@ __device__ __forceinline__ void collide_stream_cell(const StepParams<Real> &p, c
 #pragma unroll
     for (int a = 0; a < D; ++a) {
         const Real q = og * (rho * u[a] + rho * vs[a] - Real(2) * m[a]);
-        if (D == 2 || fld.fpg_by_cell) fld.fpg[a][x] = q;
-        else if (n > 0) fld.fpg[a][s0] = q;   // see Fields
+        if (D == 2) fld.fpg[a][x] = q;
+        else if (n > 0) fld.fpg[a][fld.fpg_by_cell ? x : s0] = q;   // see Fields
         ua[a] = u[a] * inv_div;
         const Real sl = ua[a] - vs[a];
         slip2 += sl * sl;
@@ -921,11 +921,11 @@ __global__ void __launch_bounds__(256) k_export_fields(FieldExport<Real> x, long
     }
     const Real *src = a == 0 ? f.src[0] : a == 1 ? f.src[1] : f.src[2];
     if (f.stride == 0) {
-        // an occupied cell's value at its first slot; the others' is
-        // 0 (rho u + 0 - 2 m), not a number where the gas has diverged
+        // an occupied cell's value at its first slot (or the cell); the others'
+        // is 0 (rho u + 0 - 2 m), not a number where the gas has diverged
         const int s0 = x.cells.begin((int)c), s1 = x.cells.begin((int)c + 1);
         const Real q = s1 > s0 && s0 >= 0 && s0 < x.np
-                           ? src[s0]
+                           ? src[x.fpg_by_cell ? (int)c : s0]
                            : Real(0) * (x.rho[c] * (a == 0 ? x.node4[c].x : a == 1 ? x.node4[c].y : x.node4[c].z));
         out[e] = (double)q * f.scale;
         return;

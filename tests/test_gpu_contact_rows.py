@@ -2,9 +2,9 @@
 runs of cells.
 
 In 3D a run spans at most 111 cells and the blocks of a group of slots share its runs; beyond 3 runs
-(2D, FP32; 8 in FP64) or 48 (3D) a block walks for the particles left.  Two steps, each from a common start-of-step
-state: what a slot keeps from the step before must not pass for its force or spin.  Bounds as in
-test_gpu_soft_spheres.py.
+(2D, FP32; 8 in FP64) or 48 (3D) a block walks for the particles left.  Two steps, each from a
+common start-of-step state: what a slot keeps from the step before must not pass for its force or
+spin.  Bounds as in test_gpu_soft_spheres.py.
 """
 import os
 import sys
